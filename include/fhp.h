@@ -278,7 +278,8 @@ FHP_API int fhp_autotune(fhp_lattice* lattice, int32_t trial_steps, int32_t* out
  * fall back to 1 when a row does not fit a stage; automatic picks 1 for
  * lattices of fewer than 8 tiles, 4 (with exchanges every second step where
  * the strips allow it) for lattices of fewer than 2 tiles per SM whose strips
- * fit, 3 up to 24 tiles per SM and 2 above (FHP-III lattices: never 4).
+ * fit, 3 up to 24 tiles per SM (single steps: 1) and 1 above (FHP-III
+ * lattices: never 4).
  * Results are identical for every choice.  While the kernel is automatic and the temporal block 1, a
  * configuration recorded by fhp_autotune for the lattice's description takes
  * precedence. */

@@ -267,6 +267,9 @@ fhp::ForcingTable fhp::forcing_table(double p) {
     fhp::ForcingTable ft;
     unsigned long long S = one;
     ft.p_plus_1 = P + 1;
+    ft.dense = P + 1 < (1ULL << 27) ? 0u : 1u;
+    ft.pre = ft.dense ? 0u : (uint32_t)(P + 1);
+    ft.inv = P > 0 ? (uint32_t)(one / (P + 1)) : 0u;
     ft.q[0] = 0;
     for (int g = 1; g <= 32; ++g) {
         S = (unsigned long long)(((unsigned __int128)S * (one - P)) >> 32);

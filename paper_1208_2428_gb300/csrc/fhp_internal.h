@@ -25,6 +25,13 @@ struct ForcingTable {
     // P + 1 with P = round(p * 2^32): Q_K <= K (P + 1), so u >= K (P + 1)
     // proves that none of K candidates is forced (cheap exact pre-check).
     unsigned long long p_plus_1;
+    // The pre-check in 32 bits: u < K * pre is the same test for P + 1 <
+    // 2^27 (32 candidates do not overflow); for larger P (p >= 1/32, where
+    // most warps hold a forced node anyway) pre is 0 and dense is 1: every
+    // quad then takes the exact walk.
+    uint32_t pre;
+    uint32_t dense;
+    uint32_t inv;   // floor(2^32 / (P + 1)): (u * inv) >> 32 never exceeds the least g with u < Q_g, minus 1
 };
 
 struct Geometry {
@@ -76,7 +83,7 @@ struct TileArgs {
 
 // Step kernel choice: automatic, direct register loads, or the bulk-copy ring
 // (cp.async.bulk into shared memory; falls back to direct when a row does not
-// fit a stage).  Automatic picks the ring when it gets >= 2 tiles per SM.
+// fit a stage).
 // kStepRun: the ring kernel running many steps in one cooperative launch
 // (per-tile dependency counters instead of a launch per step).
 // kStepResident: lattices that fit in the SMs' shared memory stay on chip for
@@ -91,7 +98,7 @@ cudaError_t launch_step(const Geometry& g, const uint32_t* src, uint32_t* dst,
                         unsigned int* err = nullptr, int kernel = kStepAuto);
 
 // The kernel fhp_step uses for `requested`: kStepDirect, kStepRing or kStepRun
-// (launch_step itself runs kStepRing for kStepRun: one step per launch).
+// (launch_step itself runs kStepDirect for kStepRun: one step per launch).
 int resolved_step_kernel(const Geometry& g, bool has_solid, int requested);
 
 // Tiles of the ring / multi-step kernels (0 if a row does not fit a stage);

@@ -45,80 +45,84 @@ struct StepVar {
     uint32_t t_lo, t_hi;
 };
 
-// Compile-time flag carried by a value (selects code inside collide_quad).
-template <bool B>
-struct Flag {
-    static constexpr bool value = B;
-};
+// Forcing of one quad: `gate` holds the first draw of each of the four words.
+// Reached by the lanes in which a word may hold a forced node (the pre-check
+// in collide_quad); visits the lane's words that pass the exact form of that
+// check, one at a time, so that the walk's code exists once (four copies of it
+// did not stay in the instruction cache: 3104 x 1498 porous medium, p = 0.02,
+// 200 steps 1285 against 1090 us, 4096 x 1024 channel, 1000 steps 3255 against
+// 3155 us).
+__device__ __forceinline__ void force_quad(const StepArgs& a, const StepVar& v, uint32_t q, uint32_t y_key, uint4 gate,
+                                           uint4 sd, uint4& o2, uint4& o5) {
+    const uint4 cand = make_uint4(o5.x & ~(o2.x | sd.x), o5.y & ~(o2.y | sd.y), o5.z & ~(o2.z | sd.z),
+                                  o5.w & ~(o2.w | sd.w));
+    uint32_t todo = 0;
+    if (gate.x < (unsigned long long)__popc(cand.x) * a.ft.p_plus_1) todo |= 1u;
+    if (gate.y < (unsigned long long)__popc(cand.y) * a.ft.p_plus_1) todo |= 2u;
+    if (gate.z < (unsigned long long)__popc(cand.z) * a.ft.p_plus_1) todo |= 4u;
+    if (gate.w < (unsigned long long)__popc(cand.w) * a.ft.p_plus_1) todo |= 8u;
+#pragma unroll 1
+    while (todo) {
+        const int j = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t f = forced_mask(word_of(cand, j), word_of(gate, j), a.ft, [&](uint32_t d) {
+            return word_of(rng_block(q, y_key, v.t_lo, v.t_hi, 1u + d, a.key), j);
+        });
+        const uint4 m = make_uint4(j == 0 ? f : 0u, j == 1 ? f : 0u, j == 2 ? f : 0u, j == 3 ? f : 0u);
+        o5 = make_uint4(o5.x ^ m.x, o5.y ^ m.y, o5.z ^ m.z, o5.w ^ m.w);
+        o2 = make_uint4(o2.x ^ m.x, o2.y ^ m.y, o2.z ^ m.z, o2.w ^ m.w);
+    }
+}
+
+// The pre-check of a quad's four words: false proves that no node is forced.
+__device__ __forceinline__ bool may_force(const StepArgs& a, uint4 gate, uint4 o2, uint4 o5, uint4 sd) {
+    bool walk = a.ft.dense != 0u;
+    walk |= gate.x < (uint32_t)__popc(o5.x & ~(o2.x | sd.x)) * a.ft.pre;
+    walk |= gate.y < (uint32_t)__popc(o5.y & ~(o2.y | sd.y)) * a.ft.pre;
+    walk |= gate.z < (uint32_t)__popc(o5.z & ~(o2.z | sd.z)) * a.ft.pre;
+    walk |= gate.w < (uint32_t)__popc(o5.w & ~(o2.w | sd.w)) * a.ft.pre;
+    return walk;
+}
 
 // Scattering, bounce-back and forcing of one quad (global quad index q of
 // row y at step v.t) whose movers have already been pulled (n0..n5), with
 // rest plane i6 and solid plane sd; the seven result planes go to o[0..6].
 // SAT selects the FHP-III (collision-saturated) rule set at compile time;
-// otherwise FHP-II or FHP-I by the lattice's rest-particle mask.
-//
-// Two uniform branches select code with constants in it: the rule set (one
-// per launch or batch tile), and whether any quad of the active lanes holds a
-// solid node -- most warps hold none, and their words then skip the
-// bounce-back multiplexers (the result is the same: a word without solid
-// nodes takes the fluid branch of every multiplexer).  On the 16384 x 4096
-// cylinder the two changes here (this one and the forcing pre-check below)
-// raised the multi-step kernel from 3159 to 3310 GSUPS and the 512-lattice
-// batch from 2484 to 2640; the resident kernel on the 4096 x 1024 channel
-// (p = 1e-3) went from 845 to 890.
+// otherwise FHP-II or FHP-I by the lattice's rest-particle mask (one uniform
+// branch per quad).
 //
 // Forcing: a word enters the candidate walk only if its first draw u is
 // below K (P + 1) for its K candidates, an upper bound of Q_K (the walk's
 // own first test, u < Q_K, decides exactly inside); a word without
-// candidates never enters.  The bound needs no table read, so the ~99.7 % of
-// words it rejects cost a popcount, a multiply and a compare.
+// candidates never enters.  The bound needs no table read: a popcount, a
+// 32-bit multiply and a compare per word, and one branch per quad.
 template <bool SOLID, bool FORCE, bool SAT = false>
 __device__ __forceinline__ void collide_quad(const StepArgs& a, const StepVar& v, int q, int y, uint4 n0, uint4 n1,
                                              uint4 n2, uint4 n3, uint4 n4, uint4 n5, uint4 i6, uint4 sd,
                                              uint4 (&o)[7]) {
-    const uint4 chi = rng_block((uint32_t)q, (uint32_t)(y + a.y_base), v.t_lo, v.t_hi, 0u, a.key);
-    uint4 gate = make_uint4(0u, 0u, 0u, 0u);
-    if (FORCE) gate = rng_block((uint32_t)q, (uint32_t)(y + a.y_base), v.t_lo, v.t_hi, 1u, a.key);
+    const uint32_t y_key = (uint32_t)(y + a.y_base);
+    const uint4 chi = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 0u, a.key);
 
-#define FHP_WORD(J, C, RR, S)                                                                   \
-    {                                                                                           \
-        Planes7 in{n0.C, n1.C, n2.C, n3.C, n4.C, n5.C, i6.C};                                   \
-        Planes7 out = SAT ? scatter_saturated(in, S ? sd.C : 0u, chi.C)                         \
-                          : scatter(in, S ? sd.C : 0u, chi.C, RR);                              \
-        if (FORCE) {                                                                            \
-            const uint32_t cand = (S ? ~sd.C : 0xFFFFFFFFu) & out.m5 & ~out.m2;                 \
-            const uint32_t u = gate.C;                                                          \
-            if ((unsigned long long)u < (unsigned long long)__popc(cand) * a.ft.p_plus_1) {     \
-                const uint32_t f = forced_mask(cand, u, a.ft, [&](uint32_t d) {                 \
-                    return word_of(rng_block((uint32_t)q, (uint32_t)(y + a.y_base), v.t_lo, v.t_hi, 1u + d,   \
-                                             a.key), J);                                        \
-                });                                                                             \
-                out.m5 ^= f;                                                                    \
-                out.m2 ^= f;                                                                    \
-            }                                                                                   \
-        }                                                                                       \
-        o[0].C = out.m0; o[1].C = out.m1; o[2].C = out.m2; o[3].C = out.m3;                     \
-        o[4].C = out.m4; o[5].C = out.m5; o[6].C = out.rest;                                    \
+#define FHP_WORD(RULES, C)                                                                        \
+    {                                                                                             \
+        const Planes7 in{n0.C, n1.C, n2.C, n3.C, n4.C, n5.C, i6.C};                               \
+        const Planes7 out = scatter_rules<RULES, SOLID>(in, sd.C, chi.C);                         \
+        o[0].C = out.m0; o[1].C = out.m1; o[2].C = out.m2; o[3].C = out.m3;                       \
+        o[4].C = out.m4; o[5].C = out.m5; o[6].C = out.rest;                                      \
     }
-    auto words = [&](auto solid, auto rest) {
-        constexpr bool S = decltype(solid)::value;
-        constexpr uint32_t RR = decltype(rest)::value ? 0xFFFFFFFFu : 0u;
-        FHP_WORD(0, x, RR, S)
-        FHP_WORD(1, y, RR, S)
-        FHP_WORD(2, z, RR, S)
-        FHP_WORD(3, w, RR, S)
-    };
-#undef FHP_WORD
-    // (Not for FHP-III: a second copy of its larger network measured 11 %
-    // slower on the cylinder.)
-    bool solid_here = SOLID;
-    if (SOLID && !SAT) solid_here = __any_sync(__activemask(), (sd.x | sd.y | sd.z | sd.w) != 0u);
-    if (SAT || a.rest_rules != 0u) {
-        if (solid_here) words(Flag<SOLID>{}, Flag<true>{});
-        else words(Flag<false>{}, Flag<true>{});
+#define FHP_QUAD(RULES) FHP_WORD(RULES, x) FHP_WORD(RULES, y) FHP_WORD(RULES, z) FHP_WORD(RULES, w)
+    if (SAT) {
+        FHP_QUAD(3)
+    } else if (a.rest_rules != 0u) {
+        FHP_QUAD(2)
     } else {
-        if (solid_here) words(Flag<SOLID>{}, Flag<false>{});
-        else words(Flag<false>{}, Flag<false>{});
+        FHP_QUAD(1)
+    }
+#undef FHP_QUAD
+#undef FHP_WORD
+    if (FORCE) {
+        const uint4 gate = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 1u, a.key);
+        if (may_force(a, gate, o[2], o[5], sd)) force_quad(a, v, (uint32_t)q, y_key, gate, sd, o[2], o[5]);
     }
 }
 
@@ -217,13 +221,6 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity) {
 // kernels' consumers spill registers: 2638 -> 3064 GSUPS on the 512-lattice
 // ensemble, 3306 -> 3430 for the multi-step kernel on the cylinder).
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
-    return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity);
-}
-
-// The same wait entirely out of line: for the single-step ring kernel's
-// consumers, where the inline test made the register allocation spill
-// (3370 -> 3190 GSUPS on the paper-size lattice).
-__device__ __noinline__ bool mbar_wait_bounded_call(uint64_t* bar, uint32_t parity) {
     return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity);
 }
 

@@ -23,7 +23,7 @@
 //                          tiles are in flight while 8 consumer warps compute;
 //   fhp_step_direct_kernel one quad per thread, operands loaded straight into
 //                          registers and neighbour words exchanged with
-//                          __shfl_sync (used when a row is too wide to stage).
+//                          __shfl_sync (the automatic choice for single steps).
 #include <cstdio>
 #include <mutex>
 
@@ -48,10 +48,9 @@ constexpr int kBarrierBytes = 128;      // mbarriers at the front of shared memo
 // the copies' bytes) release a stage to the consumer warps, and "empty"
 // barriers (one arrival per consumer warp) hand it back.  No block-wide
 // barrier is taken after set-up, and every wait is bounded.
-// SAT: the FHP-III rule set; its larger scattering network gets one CTA per
-// SM and the registers of two.
+// SAT: the FHP-III rule set.
 template <bool SOLID, bool FORCE, bool RAGGED, bool SAT>
-__global__ void __launch_bounds__(kTmaThreads, SAT ? 1 : 2) fhp_step_tma_kernel(const StepArgs a, const TileArgs ta) {
+__global__ void __launch_bounds__(kTmaThreads, 2) fhp_step_tma_kernel(const StepArgs a, const TileArgs ta) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);
     uint64_t* empty = full + kStages;
@@ -97,7 +96,7 @@ __global__ void __launch_bounds__(kTmaThreads, SAT ? 1 : 2) fhp_step_tma_kernel(
     const StepVar v{a.dst, a.t_lo, a.t_hi};
     for (int i = 0; i < count; ++i) {
         const int s = i % kStages;
-        if (!mbar_wait_bounded_call(&full[s], (uint32_t)((i / kStages) & 1))) {
+        if (!mbar_wait_bounded(&full[s], (uint32_t)((i / kStages) & 1))) {
             if (lane == 0 && a.err) atomicOr(a.err, 1u);
             return;
         }
@@ -131,7 +130,7 @@ struct RunArgs {
 };
 
 template <bool SOLID, bool FORCE, bool RAGGED, bool SAT>
-__global__ void __launch_bounds__(kRunThreads, SAT ? 1 : 2) fhp_run_kernel(const StepArgs a, const TileArgs ta,
+__global__ void __launch_bounds__(kRunThreads, 2) fhp_run_kernel(const StepArgs a, const TileArgs ta,
                                                                            const RunArgs ra) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);
@@ -370,10 +369,10 @@ __device__ __forceinline__ void direct_quad(const StepArgs& a, const Lane& L) {
     finish_quad<SOLID, FORCE, RAGGED, SAT>(a, v, L.q, y, m, n0, n1, n2, n3, n4, n5, i6, sd, L.active && in_range);
 }
 
-// SAT: the FHP-III rule set (its larger scattering network gets twice the
+// SAT: the FHP-III rule set (its larger scattering network gets more
 // registers).
 template <bool SOLID, bool FORCE, bool RAGGED, bool SAT>
-__global__ void __launch_bounds__(kBlock, SAT ? 2 : 4) fhp_step_direct_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(kBlock, SAT ? 3 : 4) fhp_step_direct_kernel(const StepArgs a) {
     const Lane L = map_lane(a);
     if (L.y & 1) direct_quad<SOLID, FORCE, RAGGED, true, SAT>(a, L);
     else direct_quad<SOLID, FORCE, RAGGED, false, SAT>(a, L);
@@ -558,13 +557,16 @@ int resolved_step_kernel(const Geometry& g, bool has_solid, int requested) {
         sms = g_dev[dev].sms;
     }
     // Few tiles per CTA and step: launch gaps and per-step pipeline refills
-    // dominate, so run all steps in one launch (measured on GB300: 903 vs 682
-    // GSUPS on 4096 x 1024, 235 vs 171 on 2048 x 512).  Many tiles per CTA:
-    // the per-step overhead is small and the single-step ring streams best.
-    // A lattice of a handful of tiles is faster with the direct kernel.
+    // dominate, so run all steps in one launch (measured on GB300: 984 vs 713
+    // GSUPS on 4096 x 1024, 3600 vs 3273 on 16384 x 4096).  Many tiles per CTA:
+    // the per-step overhead is small and the direct kernel streams best, with
+    // 32 warps an SM against the ring's 18: on 29,984 x 27,990 3702 GSUPS (6.9
+    // TB/s of algorithmic bytes) against the ring's 3051, on 16384 x 8192 3372
+    // against 2976 (FHP-III).  A lattice of a handful of tiles is faster with
+    // the direct kernel.
     const int ntiles = (g.H + R - 1) / R;
     if (ntiles < 8) return kStepDirect;
-    return ntiles <= 12 * 2 * sms ? kStepRun : kStepRing;
+    return ntiles <= 12 * 2 * sms ? kStepRun : kStepDirect;
 }
 
 int run_tiles(const Geometry& g, bool has_solid) {
@@ -638,7 +640,10 @@ cudaError_t launch_step(const Geometry& g, const uint32_t* src, uint32_t* dst,
     a.ft = ft;
     const bool ragged = (g.Wq % 4) != 0;
     const int R = tile_rows(g, has_solid);
-    if (resolved_step_kernel(g, has_solid, kernel) != kStepDirect) {
+    // (A lattice the multi-step kernel would run takes a single step with the
+    // direct kernel: 8192 x 4096 3270 against the ring's 2807 GSUPS, 4096 x 1024
+    // 713 against 681.)
+    if (resolved_step_kernel(g, has_solid, kernel) == kStepRing) {
         TileArgs ta;
         ta.R = R;
         ta.ntiles = (g.H + R - 1) / R;
