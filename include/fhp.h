@@ -244,7 +244,8 @@ FHP_API int fhp_get_temporal_block(const fhp_lattice* lattice);
  * wavefronts, 2 = 2-D tiles; a kernel that does not support the lattice or k
  * falls back to the other one.  Results are identical for every choice.
  * FHP_EINVAL for other values.  fhp_get_temporal_block_kernel returns the
- * kernel fhp_step will use for the current settings: 1 or 2, 0 when no
+ * kernel fhp_step will use for the current settings: 1 or 2, 3 where the
+ * automatic choice is register marching (see fhp_set_step_kernel), 0 when no
  * blocked pass runs (k = 1, or the resident kernel), -1 for NULL. */
 FHP_API int fhp_set_temporal_block_kernel(fhp_lattice* lattice, int32_t kind);
 FHP_API int fhp_get_temporal_block_kernel(const fhp_lattice* lattice);
@@ -266,6 +267,12 @@ FHP_API int fhp_get_temporal_block_kernel(const fhp_lattice* lattice);
 FHP_API int fhp_autotune(fhp_lattice* lattice, int32_t trial_steps, int32_t* out_kernel,
                          int32_t* out_temporal_block);
 
+/* Diagnostic: n steps (a multiple of k) as passes of k = 2 or 3 steps by
+ * register marching, the kernel the automatic choice uses on large lattices
+ * (see fhp_set_step_kernel), on a lattice of any size with H >= 2k + 2;
+ * FHP_EINVAL otherwise.  Results are those of fhp_step. */
+FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
+
 /* Step kernel used by fhp_step: 0 = automatic (default), 4 = shared-memory
  * resident (the lattice is cut into one strip per SM and stays in shared
  * memory for all steps of a call; only the strips' edge rows are exchanged
@@ -280,6 +287,12 @@ FHP_API int fhp_autotune(fhp_lattice* lattice, int32_t trial_steps, int32_t* out
  * the strips allow it) for lattices of fewer than 2 tiles per SM whose strips
  * fit, 3 up to 24 tiles per SM (single steps: 1) and 1 above (FHP-III
  * lattices: never 4).
+ * Lattices of 12 million nodes and more (40 million with forcing, whose
+ * probability must be below 0.0025; 200 million for forced FHP-III lattices)
+ * instead run passes of 2 or 3 steps by register marching -- every lane of a
+ * warp marches a column of 128-node quads up a band of rows with the
+ * intermediate time levels in registers, all passes of a call in one
+ * cooperative launch -- and only the remaining step by these kernels.
  * Results are identical for every choice.  While the kernel is automatic and the temporal block 1, a
  * configuration recorded by fhp_autotune for the lattice's description takes
  * precedence. */

@@ -65,7 +65,7 @@ struct TuneKey {
 struct TuneChoice {
     int kernel;   // fhp::StepKernel other than kStepAuto
     int k;        // temporal block
-    int bk;       // temporal-block kernel (0 automatic, 1 row wavefronts, 2 tiles)
+    int bk;       // temporal-block kernel (0 automatic, 1 row wavefronts, 2 tiles, 3 register marching)
 };
 std::mutex g_tune_mutex;
 std::vector<std::pair<TuneKey, TuneChoice>> g_tuned;
@@ -162,7 +162,8 @@ struct DeviceGuard {
 
 // Kernel and temporal block fhp_step uses: the lattice's own settings, or,
 // while they are automatic (kernel 0, k = 1), the configuration autotuned
-// for this shape if there is one, else the shared-memory resident kernel
+// for this shape if there is one, else register marching for the lattices it
+// is fastest on (fhp::march_choice), else the shared-memory resident kernel
 // (exchanging every second step where the strips allow it) for lattices it
 // holds whose multi-step ring would give fewer than two tiles per SM
 // (launch-bound sizes, where it measured fastest: 1163 vs 957 GSUPS on
@@ -177,6 +178,11 @@ void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk
         *kernel = c.kernel;
         *k_block = c.k;
         if (bk) *bk = c.bk;
+        return;
+    }
+    if (const int mk = fhp::march_choice(h->g, h->ft, h->force)) {
+        *k_block = mk;
+        if (bk) *bk = 3;
         return;
     }
     const int resolved = fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepAuto);
@@ -201,12 +207,14 @@ int resident_interval(const fhp_lattice* h, int kernel, int k_block) {
 // Kernel of a temporally blocked pass of k steps for the requested kind
 // (0 automatic, 1 row wavefronts, 2 tiles): 1 or 2, the other one where the
 // requested kernel does not support the lattice, 0 if neither does (k = 1).
+// (3, register marching, is only ever chosen by the library.)
 // Automatic takes the 2-D tiles where they apply: on GB300 they measured
 // faster than the row wavefronts on every lattice tried (16384 x 4096,
 // k = 2: 1815 against 1175 GSUPS), whose per-row hand-offs between warps
 // leave most warps waiting.
 int blocked_kind(const fhp_lattice* h, int k, int bk) {
     if (k <= 1) return 0;
+    if (bk == 3) return fhp::march_supported(h->g, k) ? 3 : 0;
     const bool wave = fhp::wave_supported(h->g, k), tiles = fhp::block_supported(h->g, k);
     if (bk == 1) return wave ? 1 : (tiles ? 2 : 0);
     return tiles ? 2 : (wave ? 1 : 0);
@@ -470,6 +478,39 @@ struct NvtxRange {
 };
 }  // namespace
 
+namespace {
+// Register marching: as many of *n steps as passes of k (and one of 2 for a
+// remainder of 2) cover; *n is left with the others.  The passes' counters
+// live in the byte-staging area.
+int march_steps(fhp_lattice* h, int k, int64_t* n) {
+    const fhp::Key2 key{(uint32_t)h->seed, (uint32_t)(h->seed >> 32)};
+    for (; k >= 2; --k)
+        while (*n >= k) {
+            const int64_t most = *n / k;
+            const int passes = (int)(most < (1 << 20) ? most : (1 << 20));
+            cudaError_t e = fhp::launch_march(h->g, h->buf[h->cur], h->buf[h->cur ^ 1], h->solid, h->has_solid, h->force,
+                                              h->ft, key, (uint64_t)h->t, k, passes,
+                                              reinterpret_cast<unsigned int*>(h->staging), h->staging_bytes,
+                                              h->stream, h->flags + 1);
+            if (e != cudaSuccess) return cuda_fail(h, e, "launching the register-marching kernel");
+            ++h->launches;
+            h->cur ^= passes & 1;
+            h->t += (int64_t)passes * k;
+            *n -= (int64_t)passes * k;
+        }
+    return FHP_OK;
+}
+}  // namespace
+
+int fhp_step_march(fhp_lattice* h, int32_t k, int64_t n) {
+    if (!h) return fail(nullptr, FHP_EINVAL, "lattice is NULL");
+    if (n < 0 || n > kMaxTime - h->t) return fail(h, FHP_EINVAL, "step count %lld out of range", (long long)n);
+    if ((k != 2 && k != 3) || n % k || !fhp::march_supported(h->g, k))
+        return fail(h, FHP_EINVAL, "passes of %d steps do not cover %lld steps of this lattice", k, (long long)n);
+    DeviceGuard dg(h->device);
+    return march_steps(h, k, &n);
+}
+
 int fhp_step(fhp_lattice* h, int64_t n) {
     NvtxRange nvtx("fhp_step");
     if (!h) return fail(nullptr, FHP_EINVAL, "lattice is NULL");
@@ -501,7 +542,10 @@ int fhp_step(fhp_lattice* h, int64_t n) {
     }
     if (kernel == fhp::kStepResident) kernel = fhp::kStepAuto;  // not supported for this lattice
     const int blocked = blocked_kind(h, k_block, bk);
-    if (blocked != 0) {
+    if (blocked == 3) {
+        const int rc = march_steps(h, k_block, &n);
+        if (rc != FHP_OK) return rc;
+    } else if (blocked != 0) {
         const bool wave = blocked == 1;
         // Temporal blocking: passes of k steps (row wavefronts where the rows
         // fit shared memory, else 2-D tiles); the remainder one step at a time.
@@ -744,6 +788,11 @@ int fhp_autotune(fhp_lattice* h, int32_t trial_steps, int32_t* out_kernel, int32
         if (fhp::wave_supported(h->g, k)) cands.push_back({fhp::kStepDirect, k, 1});
     for (int k : {2, 4, 8})
         if (fhp::block_supported(h->g, k)) cands.push_back({fhp::kStepDirect, k, 2});
+    // Register marching (remainders on the ring kernel where a row fits it).
+    const int rest_kernel = fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepRing);
+    const int mk = fhp::march_choice(h->g, h->ft, h->force);
+    if (mk == 2 || (h->g.rules != 3 && fhp::march_supported(h->g, 2))) cands.push_back({rest_kernel, 2, 3});
+    if (mk == 3) cands.push_back({rest_kernel, 3, 3});
     TuneChoice best{fhp::kStepDirect, 1, 0};
     float best_ms = -1.0f;
     for (size_t i = 0; e == cudaSuccess && i < cands.size(); ++i) {

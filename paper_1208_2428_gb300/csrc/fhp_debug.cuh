@@ -30,6 +30,8 @@ enum DebugSite : unsigned int {
     kSiteBatchBlockHeader = 10, // batch temporal blocking: a tile within its member, its rows within a plane
     kSiteBatchBlockStage = 11,  // ... the rows of a bulk copy within the staged plane
     kSiteBatchBlockQuad = 12,   // ... the rows and words a quad reads
+    kSiteMarchLoad = 13,     // register marching: a loaded quad within its plane
+    kSiteMarchStore = 14,    // ... a stored quad within its plane
     kSiteSelfTest = 99,      // fhp_debug_selftest
 };
 

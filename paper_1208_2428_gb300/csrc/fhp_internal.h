@@ -171,6 +171,21 @@ cudaError_t launch_wave(const Geometry& g, const uint32_t* src, uint32_t* dst, c
                         bool has_solid, bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int k,
                         cudaStream_t stream, unsigned int* err);
 
+// Temporal blocking in registers (fhp_march.cu): `passes` passes of k (2 or 3)
+// steps from src (state at t0); the result is in dst if `passes` is odd, else
+// in src.  Every lane marches a quad column up a band of rows; all passes run
+// in one cooperative launch, a warp waiting only for the warps around it.  Any
+// rule set and row width; needs H >= 2k + 2 and planes of less than 4 GiB.
+// `flags` is scratch of `flag_bytes` (a word per warp; too few: one launch per
+// pass).
+bool march_supported(const Geometry& g, int k);
+// Steps per pass for which register marching is the automatic choice (0: it
+// is not).
+int march_choice(const Geometry& g, const ForcingTable& ft, bool force);
+cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const uint32_t* solid, bool has_solid,
+                         bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int k, int passes,
+                         unsigned int* flags, size_t flag_bytes, cudaStream_t stream, unsigned int* err);
+
 // Pack H x W node bytes (device) into 7 state planes + the solid plane.
 // Sets *device_any_solid to a nonzero value if any node is solid.
 cudaError_t launch_pack(const Geometry& g, const uint8_t* bytes, uint32_t* state,

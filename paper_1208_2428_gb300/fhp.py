@@ -86,6 +86,7 @@ def load(path: str | None = None):
         "fhp_get_state_device": (ctypes.c_int, [vp, u8p]),
         "fhp_load_obstacles": (ctypes.c_int, [vp, u8p]),
         "fhp_step": (ctypes.c_int, [vp, i64]),
+        "fhp_step_march": (ctypes.c_int, [vp, i32, i64]),
         "fhp_coarse_grain": (ctypes.c_int, [vp, i32, vp, vp, vp, vp]),
         "fhp_coarse_grain_device": (ctypes.c_int, [vp, i32, vp, vp, vp, vp]),
         "fhp_get_time": (i64, [vp]),
@@ -283,6 +284,10 @@ class Lattice:
     def step(self, n: int = 1):
         self._check(self._lib.fhp_step(self._h, int(n)))
 
+    def step_march(self, k: int, n: int):
+        """Diagnostic: n steps as register-marching passes of k = 2 or 3 steps (see fhp.h)."""
+        self._check(self._lib.fhp_step_march(self._h, int(k), int(n)))
+
     @property
     def t(self) -> int:
         return int(self._lib.fhp_get_time(self._h))
@@ -303,7 +308,7 @@ class Lattice:
 
     @property
     def temporal_block_kernel(self) -> int:
-        """Kernel of the blocked passes fhp_step runs: 1 wavefronts, 2 tiles, 0 none."""
+        """Kernel of the blocked passes fhp_step runs: 1 wavefronts, 2 tiles, 3 register marching, 0 none."""
         return int(self._lib.fhp_get_temporal_block_kernel(self._h))
 
     def set_step_kernel(self, kind: int):

@@ -1,0 +1,92 @@
+"""Register marching (passes of 2 or 3 steps with the intermediate time levels
+in registers): bit-exact with the oracle on every way columns are dealt to
+lanes and rows to bands, and the automatic choice of it with the direct step
+kernel."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1208_2428_gb300 import build as cuda_build
+    cuda_build.build()
+    import paper_1208_2428_gb300 as p
+    p.load()
+    return p
+
+
+# Whole rows in a warp (1, 2, 3, 16, 32 quads; partial last quads) and chains
+# of columns cut every 30 or 28 lanes (33 and more quads; last quads of 1, 2,
+# 3 and 4 words); heights of one band, of several, and with a short last band.
+SIZES = [(32, 8), (96, 14), (256, 26), (352, 10), (2048, 14), (3968, 8), (4096, 38), (4128, 10), (4160, 14),
+         (4192, 26), (4224, 8), (8192, 22), (8224, 14), (29984, 10)]
+
+
+@pytest.mark.parametrize("k", [2, 3])
+@pytest.mark.parametrize("W,H", SIZES)
+@pytest.mark.parametrize("variant", ["periodic", "walls_rare", "points_dense", "fhp1", "fhp3"])
+def test_march_matches_oracle(pkg, oracle_mod, W, H, k, variant):
+    seed = 31 * W + H + k
+    rng = np.random.Generator(np.random.PCG64(seed))
+    solid, p, rules = {"periodic": (None, 0.0, 2), "walls_rare": (workloads.channel_walls(W, H), 0.02, 2),
+                       "points_dense": (workloads.random_points(W, H, 0.05, rng), 0.3, 2),
+                       "fhp1": (workloads.channel_walls(W, H), 0.0, 1),
+                       "fhp3": (None, 0.01, 3)}[variant]
+    s0 = workloads.bernoulli_lattice(W, H, 0.35, seed, solid)
+    with pkg.Lattice(W, H, seed=seed, forcing_p=p) as lat:
+        lat.set_rules(rules)
+        lat.set_state(s0)
+        lat.set_time(2**32 - 5)          # the steps pass a carry of the time counter
+        lat.step_march(k, k)             # one pass: no waits
+        lat.step_march(k, 6 * k)         # passes that wait for one another
+        got = lat.get_state()
+        assert lat.t == 2**32 - 5 + 7 * k
+    want, _ = oracle_mod.run(s0, seed, 2**32 - 5, 7 * k, p, rules=rules)
+    assert np.array_equal(got, want), f"{int((got != want).sum())} nodes differ"
+
+
+def test_march_every_candidate_forced_and_full(pkg, oracle_mod):
+    W, H = 4160, 12
+    for fill in (0x7F, 0x20, 0xFF):
+        s0 = np.full((H, W), fill, dtype=np.uint8)
+        with pkg.Lattice(W, H, seed=9, forcing_p=1.0) as lat:
+            lat.set_state(s0)
+            lat.step_march(2, 8)
+            got = lat.get_state()
+        want, _ = oracle_mod.run(s0, 9, 0, 8, 1.0)
+        assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("W,H,p,block", [(4096, 4096, 0.0, 3), (8192, 4096, 0.0, 2), (16384, 2560, 5e-4, 2),
+                                         (12032, 3400, 1e-3, 2)])
+def test_automatic_choice_equals_direct_kernel(pkg, W, H, p, block):
+    import torch
+    got = []
+    for kernel in (0, 1):
+        with pkg.Lattice(W, H, seed=5, forcing_p=p, step_kernel=kernel) as lat:
+            lat.load_obstacle_shapes(workloads.cylinder_shapes(W, H))
+            lat.init_random(0.3)
+            if kernel == 0:
+                assert lat.temporal_block_kernel == 3 and lat.temporal_block == block
+            lat.step(17)
+            got.append(lat.get_state_tensor())
+            lat.synchronize()
+    assert torch.equal(got[0], got[1])
+
+
+def test_march_refusals(pkg):
+    with pkg.Lattice(64, 6, seed=1) as lat:
+        lat.step_march(2, 0)
+        for k, n in [(1, 2), (4, 4), (2, 3), (3, 6), (2, -2)]:   # (k = 3 needs 8 rows)
+            with pytest.raises(pkg.FhpError):
+                lat.step_march(k, n)
+        assert lat.t == 0
