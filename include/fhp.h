@@ -282,17 +282,16 @@ FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
  * cp.async.bulk, one launch per step), 3 = multi-step ring (the ring kernel
  * running all steps of an fhp_step call in one cooperative launch, each tile
  * waiting only for the three tiles of the previous step it reads).  2 and 3
- * fall back to 1 when a row does not fit a stage; automatic picks 1 for
- * lattices of fewer than 8 tiles, 4 (with exchanges every second step where
- * the strips allow it) for lattices of fewer than 2 tiles per SM whose strips
- * fit, 3 up to 24 tiles per SM (single steps: 1) and 1 above (FHP-III
- * lattices: never 4).
- * Lattices of 12 million nodes and more (40 million with forcing, whose
- * probability must be below 0.0025; 200 million for forced FHP-III lattices)
- * instead run passes of 2 or 3 steps by register marching -- every lane of a
- * warp marches a column of 128-node quads up a band of rows with the
- * intermediate time levels in registers, all passes of a call in one
- * cooperative launch -- and only the remaining step by these kernels.
+ * fall back to 1 when a row does not fit a stage.  Automatic picks 4 for
+ * lattices whose strips fit (calls of up to three steps: 1; FHP-III lattices:
+ * never 4), else register marching for lattices of 12 million nodes and more
+ * (40 million with forcing, whose probability must be below 0.0025; 200
+ * million for forced FHP-III lattices): passes of 2 or 3 steps in which every
+ * lane of a warp marches a column of 128-node quads up a band of rows with
+ * the intermediate time levels in registers, all passes of a call in one
+ * cooperative launch, and only a remaining step runs on the kernels below.
+ * Else it picks 1 for lattices of fewer than 8 tiles, 3 up to 24 tiles per SM
+ * (single steps: 1) and 1 above.
  * Results are identical for every choice.  While the kernel is automatic and the temporal block 1, a
  * configuration recorded by fhp_autotune for the lattice's description takes
  * precedence. */

@@ -162,12 +162,12 @@ struct DeviceGuard {
 
 // Kernel and temporal block fhp_step uses: the lattice's own settings, or,
 // while they are automatic (kernel 0, k = 1), the configuration autotuned
-// for this shape if there is one, else register marching for the lattices it
-// is fastest on (fhp::march_choice), else the shared-memory resident kernel
-// (exchanging every second step where the strips allow it) for lattices it
-// holds whose multi-step ring would give fewer than two tiles per SM
-// (launch-bound sizes, where it measured fastest: 1163 vs 957 GSUPS on
-// 4096 x 1024, 1979 vs 1573 on 4096 x 2048).
+// for this shape if there is one, else the shared-memory resident kernel for
+// every lattice it holds (us a step, p = 1e-3, against the multi-step ring: 512 x
+// 512 1.6 against 4.4, 4096 x 1024 1.9 against 4.2, 4096 x 3072 3.3 against 5.5,
+// 4096 x 4096 3.7 against register marching's 5.7), else register marching for the lattices it
+// is fastest on (fhp::march_choice), else the kernel of
+// fhp::resolved_step_kernel.
 void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk = nullptr) {
     *kernel = h->step_kernel;
     *k_block = h->k_block;
@@ -180,19 +180,13 @@ void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk
         if (bk) *bk = c.bk;
         return;
     }
+    if (fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 1)) {
+        *kernel = fhp::kStepResident;
+        return;
+    }
     if (const int mk = fhp::march_choice(h->g, h->ft, h->force)) {
         *k_block = mk;
         if (bk) *bk = 3;
-        return;
-    }
-    const int resolved = fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepAuto);
-    const int tiles = fhp::run_tiles(h->g, h->has_solid);
-    int dev_sms = 0;
-    if (resolved == fhp::kStepRun && cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, h->device) ==
-                                         cudaSuccess &&
-        tiles < 2 * dev_sms && fhp::resident_supported(h->g, h->has_solid, h->staging_bytes)) {
-        *kernel = fhp::kStepResident;
-        *k_block = fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 2) ? 2 : 1;
     }
 }
 
@@ -520,7 +514,14 @@ int fhp_step(fhp_lattice* h, int64_t n) {
     const fhp::Key2 key{(uint32_t)h->seed, (uint32_t)(h->seed >> 32)};
     int kernel = h->step_kernel, k_block = h->k_block, bk = h->block_kernel;
     effective_settings(h, &kernel, &k_block, &bk);
-    const int gh = resident_interval(h, kernel, k_block);
+    int gh = resident_interval(h, kernel, k_block);
+    if (gh > 0 && n <= 3 && h->step_kernel == fhp::kStepAuto) {
+        // Up to three steps do not repay moving the lattice into shared memory
+        // and back (about 10 us; a direct step of such a lattice takes 4 to 6).
+        gh = 0;
+        kernel = fhp::kStepDirect;
+        k_block = 1;
+    }
     if (gh > 0) {
         // The lattice stays in shared memory for launches of up to 2^24 steps
         // (exchange rows in the byte-staging area, step counters in the tile

@@ -121,7 +121,7 @@ cudaError_t launch_run(const Geometry& g, uint32_t* buf0, uint32_t* buf1, const 
 // (state at t0); the result is in buf0 if n is even, else in buf1.  `halo`
 // needs resident_halo_words() words, `flags` one word per SM (both scratch).
 bool resident_supported(const Geometry& g, bool has_solid, size_t staging_bytes, int gh = 1);
-size_t resident_halo_words(const Geometry& g, int gh);
+size_t resident_halo_words(const Geometry& g, bool has_solid, int gh);
 cudaError_t launch_resident(const Geometry& g, uint32_t* buf0, uint32_t* buf1, const uint32_t* solid, bool has_solid,
                             bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int nsteps, int gh,
                             uint32_t* halo, unsigned int* flags, cudaStream_t stream, unsigned int* err);

@@ -96,12 +96,12 @@ __device__ __forceinline__ bool may_force(const StepArgs& a, uint4 gate, uint4 o
 // own first test, u < Q_K, decides exactly inside); a word without
 // candidates never enters.  The bound needs no table read: a popcount, a
 // 32-bit multiply and a compare per word, and one branch per quad.
+// (collide_drawn takes the quad's random blocks from the caller: chirality
+// `chi`, first forcing draws `gate`.)
 template <bool SOLID, bool FORCE, bool SAT = false>
-__device__ __forceinline__ void collide_quad(const StepArgs& a, const StepVar& v, int q, int y, uint4 n0, uint4 n1,
-                                             uint4 n2, uint4 n3, uint4 n4, uint4 n5, uint4 i6, uint4 sd,
-                                             uint4 (&o)[7]) {
-    const uint32_t y_key = (uint32_t)(y + a.y_base);
-    const uint4 chi = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 0u, a.key);
+__device__ __forceinline__ void collide_drawn(const StepArgs& a, const StepVar& v, int q, int y, uint4 chi, uint4 gate,
+                                              uint4 n0, uint4 n1, uint4 n2, uint4 n3, uint4 n4, uint4 n5, uint4 i6,
+                                              uint4 sd, uint4 (&o)[7]) {
 
 #define FHP_WORD(RULES, C)                                                                        \
     {                                                                                             \
@@ -120,10 +120,19 @@ __device__ __forceinline__ void collide_quad(const StepArgs& a, const StepVar& v
     }
 #undef FHP_QUAD
 #undef FHP_WORD
-    if (FORCE) {
-        const uint4 gate = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 1u, a.key);
-        if (may_force(a, gate, o[2], o[5], sd)) force_quad(a, v, (uint32_t)q, y_key, gate, sd, o[2], o[5]);
-    }
+    if (FORCE && may_force(a, gate, o[2], o[5], sd))
+        force_quad(a, v, (uint32_t)q, (uint32_t)(y + a.y_base), gate, sd, o[2], o[5]);
+}
+
+template <bool SOLID, bool FORCE, bool SAT = false>
+__device__ __forceinline__ void collide_quad(const StepArgs& a, const StepVar& v, int q, int y, uint4 n0, uint4 n1,
+                                             uint4 n2, uint4 n3, uint4 n4, uint4 n5, uint4 i6, uint4 sd,
+                                             uint4 (&o)[7]) {
+    const uint32_t y_key = (uint32_t)(y + a.y_base);
+    const uint4 chi = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 0u, a.key);
+    uint4 gate = make_uint4(0u, 0u, 0u, 0u);
+    if (FORCE) gate = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 1u, a.key);
+    collide_drawn<SOLID, FORCE, SAT>(a, v, q, y, chi, gate, n0, n1, n2, n3, n4, n5, i6, sd, o);
 }
 
 // Store a quad's seven result planes to global memory (the padding words of

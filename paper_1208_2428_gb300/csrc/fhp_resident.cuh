@@ -14,17 +14,20 @@ namespace fhp {
 
 constexpr int kResThreads = 384;   // 12 warps: 3 per SM sub-partition at <= 168 registers
                                    // (both kernels use at most 160: no spills)
-constexpr int kResSmemLimit = 220 * 1024;
+constexpr int kRes1Threads = 512;  // one-row exchange: 16 warps at <= 128 registers
+constexpr int kResSmemLimit = 224 * 1024;
 
 struct ResArgs {
     uint32_t* buf0;        // state at t0; also the result when nsteps is even
     uint32_t* buf1;        // the result when nsteps is odd
-    uint32_t* halo;        // exchange rows: [2 parities][G][2 sides][row planes][Pq] words (2 row
-                           // planes per side for the one-row exchange, 9 for two ghost rows)
-    unsigned int* flags;   // [G] step counters, zero at launch
+    uint32_t* halo;        // exchange rows.  Two ghost rows: [2 parities][G][2 sides][9 row planes][Pq]
+                           // words.  One row: [2 parities][G][2 sides][2 planes][nq] units of 32 bytes,
+                           // zero at launch
+    unsigned int* flags;   // two ghost rows: [G] step counters, zero at launch
     int nsteps;
     unsigned long long t0;
     int nmax;              // most rows any CTA owns
+    unsigned long long nq_magic;   // ceil(2^32 / nq): j / nq == (j * nq_magic) >> 32 for small j
 };
 
 // Launches the two-ghost-row kernel (fhp_resident_ghost.cu) for the
@@ -35,7 +38,7 @@ cudaError_t launch_resident_ghost2(const StepArgs& a, const ResArgs& ra, int gri
 // Sets the dynamic shared-memory limit of `fn` once per device and launches
 // it cooperatively with the kernel arguments (a, ra).
 cudaError_t launch_resident_coop(const void* fn, bool* configured, const StepArgs& a, const ResArgs& ra, int grid,
-                                 size_t smem, cudaStream_t s);
+                                 int threads, size_t smem, cudaStream_t s);
 
 namespace {
 
@@ -70,10 +73,11 @@ __device__ __noinline__ bool wait_neighbours(const unsigned int* flags, int p, i
 // movers from the staged rows of `src`, scatters, and writes the seven planes
 // of the new state into `dst` (padding words of a ragged row stay zero).
 // (Local row lr of the staged buffers, lattice row y, `Srow` its solid row.)
+// (resident_quad_drawn takes the quad's random blocks from the caller.)
 template <bool SOLID, bool FORCE, bool RAGGED>
-__device__ __forceinline__ void resident_quad_at(const StepArgs& a, const StepVar& v, const uint32_t* src,
-                                                 uint32_t* dst, const uint32_t* Srow, size_t pstride, int lr, int y,
-                                                 int q, uint4 (&o)[7]) {
+__device__ __forceinline__ void resident_quad_drawn(const StepArgs& a, const StepVar& v, const uint32_t* src,
+                                                    uint32_t* dst, const uint32_t* Srow, size_t pstride, int lr, int y,
+                                                    int q, uint4 chi, uint4 gate, uint4 (&o)[7]) {
     const int Pq = a.Pq;
     const int w = 4 * q;
     const int m = RAGGED ? (q == a.nq - 1 ? a.Wq - w : 4) : 4;
@@ -104,7 +108,7 @@ __device__ __forceinline__ void resident_quad_at(const StepArgs& a, const StepVa
         n3 = i3;
         n1 = i1;
     }
-    collide_quad<SOLID, FORCE>(a, v, q, y, n0, n1, n2, n3, n4, n5, i6, sd, o);
+    collide_drawn<SOLID, FORCE>(a, v, q, y, chi, gate, n0, n1, n2, n3, n4, n5, i6, sd, o);
     if (RAGGED && m < 4) {
 #pragma unroll
         for (int k = 0; k < 7; ++k) {
@@ -115,6 +119,23 @@ __device__ __forceinline__ void resident_quad_at(const StepArgs& a, const StepVa
     }
 #pragma unroll
     for (int k = 0; k < 7; ++k) st4(dst + k * pstride + (size_t)lr * Pq + w, o[k]);
+}
+
+template <bool FORCE>
+__device__ __forceinline__ void resident_draws(const StepArgs& a, const StepVar& v, int q, int y, uint4& chi,
+                                               uint4& gate) {
+    const uint32_t y_key = (uint32_t)(y + a.y_base);
+    chi = rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 0u, a.key);
+    gate = FORCE ? rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 1u, a.key) : make_uint4(0u, 0u, 0u, 0u);
+}
+
+template <bool SOLID, bool FORCE, bool RAGGED>
+__device__ __forceinline__ void resident_quad_at(const StepArgs& a, const StepVar& v, const uint32_t* src,
+                                                 uint32_t* dst, const uint32_t* Srow, size_t pstride, int lr, int y,
+                                                 int q, uint4 (&o)[7]) {
+    uint4 chi, gate;
+    resident_draws<FORCE>(a, v, q, y, chi, gate);
+    resident_quad_drawn<SOLID, FORCE, RAGGED>(a, v, src, dst, Srow, pstride, lr, y, q, chi, gate, o);
 }
 
 // One step's work items in two classes: the edge items (the rows the

@@ -167,7 +167,7 @@ cudaError_t launch_ghost_variant(const StepArgs& a, const ResArgs& ra, int grid,
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     return launch_resident_coop((const void*)fhp_resident_ghost_kernel<SOLID, FORCE, RAGGED, 2>,
-                                &g_ghost_configured[dev][SOLID][FORCE][RAGGED], a, ra, grid, smem, s);
+                                &g_ghost_configured[dev][SOLID][FORCE][RAGGED], a, ra, grid, kResThreads, smem, s);
 }
 
 }  // namespace
