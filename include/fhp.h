@@ -417,8 +417,10 @@ FHP_API int fhp_batch_step(fhp_batch* batch, int64_t n);
  * batch's stream after the one-time set-up of every candidate (graph
  * capture, device tables, kernel attributes), and a later call records the
  * candidate with the most node updates per millisecond for the class (read
- * without waiting); until then SINGLE_STEP with 256-quad tiles and no
- * blocking runs.  Results are identical for every choice. */
+ * without waiting); until then, while the temporal block is automatic too,
+ * register marching runs (see fhp_batch_set_temporal_block), else
+ * SINGLE_STEP with 256-quad tiles and no blocking.  Results are identical for
+ * every choice. */
 #define FHP_BATCH_KERNEL_AUTO 0
 #define FHP_BATCH_KERNEL_SINGLE_STEP 1
 #define FHP_BATCH_KERNEL_MULTI_STEP 2
@@ -452,10 +454,15 @@ FHP_API int32_t fhp_batch_tile_count(fhp_batch* batch);
  * remaining steps (s mod k, all s for wider members) run on the batch step
  * kernel.  Every member's state equals s single steps bit for bit.
  * k = 1: no blocking.  k = 0 (default): automatic -- while the step kernel is
- * AUTO, blocked passes of k = 2 and k = 4 (remainders on the single-step
- * kernel) join the online tuning trial as two more candidates (c = 6, or 4
- * with a fixed tile size) and the fastest candidate's temporal block is
- * recorded with its kernel; otherwise none.  FHP_EINVAL for other values.
+ * AUTO, register marching (all passes of 2 or 3 steps of a call in one
+ * cooperative launch, members of any width with at least 6 rows and a forcing
+ * probability below 0.01; the other members and remaining single steps on the
+ * single-step kernel) and blocked passes of k = 4 join the online tuning trial
+ * as two more candidates (c = 6, or 4 with a fixed tile size) and the fastest
+ * candidate's temporal block is recorded with its kernel (2 or 3: register
+ * marching); otherwise none.  FHP_EINVAL for other values.
+ * Register marching takes 10 KB from the arena while there is room and gives
+ * them up to any other use.
  * Blocked passes take a descriptor table (about 0.4 KB per member slot) and
  * a tile list (12 bytes per tile) from the arena: with k = 2 or 4 a call
  * fails with FHP_ENOMEM if the arena cannot hold them; the automatic choice

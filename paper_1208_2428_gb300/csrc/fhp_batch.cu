@@ -455,6 +455,7 @@ struct Member {
     int64_t steps_left = -1;      // -1: no budget
     bool has_solid = false;
     int R = 1;
+    fhp::MarchLayout lay[2] = {}; // register marching, k = 2 and 3
     int tile_base = 0;            // first entry of the member's tiles in the tile list
 };
 
@@ -493,6 +494,7 @@ struct TuneTrial {
     int kind[kTuneCands] = {};
     int quads[kTuneCands] = {};
     int block[kTuneCands] = {};      // temporal block k (1: none)
+    bool march[kTuneCands] = {};     // ... as register marching
     cudaEvent_t ev[kTuneCands][2] = {};   // [candidate][start, end]
     double updates[kTuneCands] = {};
 };
@@ -515,6 +517,10 @@ struct fhp_batch {
     int tuned[kTuneClasses] = {};               // per tile-count class: kernel measured fastest (0: unknown)
     int tuned_quads[kTuneClasses] = {};         // ... and its tile size (quads per tile)
     int tuned_block[kTuneClasses] = {};         // ... and its temporal block (1: none)
+    bool tuned_march[kTuneClasses] = {};        // ... run as register marching
+    unsigned int* d_march_flags = nullptr;      // register marching: pass counters (from the arena, on demand)
+    unsigned int march_epoch = 0;               // no counter is above this
+    std::vector<fhp::MarchBatch> h_march;       // its member table (one entry, on demand)
     int tile_quads = 0;                         // quads per tile: 0 automatic (tuned with the kernel)
     int temporal_block = 0;                     // 0 automatic (tuned with the kernel), 1 none, 2 or 4
     // blocked passes: member table and tile list (allocated from the arena)
@@ -570,11 +576,26 @@ size_t tile_table_bytes(size_t cap) {
     return fhp::round256(cap * sizeof(fhp::BatchTile)) + fhp::round256(cap * sizeof(unsigned int));
 }
 
+constexpr size_t kMarchFlagBytes = (size_t)fhp::kMarchMaxCtas * fhp::kMarchCtaWarps * sizeof(unsigned int);
+
+// A block of the arena (SIZE_MAX if there is no room).  The counters of
+// register marching, which a batch can do without, give way to anything else:
+// whatever takes their place is queued behind the launches that use them.
+size_t take(fhp_batch* b, size_t bytes) {
+    size_t off = b->arena.allocate(bytes);
+    if (off == SIZE_MAX && b->d_march_flags) {
+        b->arena.release((size_t)((uint8_t*)b->d_march_flags - b->arena_base), kMarchFlagBytes);
+        b->d_march_flags = nullptr;
+        off = b->arena.allocate(bytes);
+    }
+    return off;
+}
+
 // Make sure the device tables can hold `lats` lattices and `tiles` tiles.
 int ensure_tables(fhp_batch* b, size_t lats, size_t tiles) {
     if (lats > b->lat_cap) {
         const size_t cap = std::max<size_t>(lats, 2 * b->lat_cap + 16);
-        const size_t off = b->arena.allocate(cap * sizeof(fhp::BatchLattice));
+        const size_t off = take(b, cap * sizeof(fhp::BatchLattice));
         if (off == SIZE_MAX) return bfail(b, FHP_ENOMEM, "batch arena full (descriptor table)");
         if (b->lat_off != SIZE_MAX) b->arena.release(b->lat_off, b->lat_cap * sizeof(fhp::BatchLattice));
         b->lat_off = off;
@@ -585,7 +606,7 @@ int ensure_tables(fhp_batch* b, size_t lats, size_t tiles) {
     if (tiles > b->tile_cap) {
         // The tile list followed by one completion counter per tile.
         const size_t cap = std::max<size_t>(tiles, 2 * b->tile_cap + 256);
-        const size_t off = b->arena.allocate(tile_table_bytes(cap));
+        const size_t off = take(b, tile_table_bytes(cap));
         if (off == SIZE_MAX) return bfail(b, FHP_ENOMEM, "batch arena full (tile table)");
         if (b->tile_off != SIZE_MAX) b->arena.release(b->tile_off, tile_table_bytes(b->tile_cap));
         b->tile_off = off;
@@ -609,7 +630,7 @@ int rows_per_tile(const fhp::Geometry& g, int quads = kDefaultTileQuads) {
 }
 
 int scratch_bytes_op(fhp_batch* b, size_t bytes, size_t* off) {
-    *off = b->arena.allocate(bytes);
+    *off = take(b, bytes);
     if (*off == SIZE_MAX) return bfail(b, FHP_ENOMEM, "batch arena full (staging of %zu bytes)", bytes);
     return FHP_OK;
 }
@@ -700,7 +721,7 @@ int fhp_batch_add(fhp_batch* b, int32_t width, int32_t height, uint64_t seed, do
     m.p = forcing_p;
     m.ft = fhp::forcing_table(forcing_p);
     m.bytes = member_bytes(g);
-    m.off = b->arena.allocate(m.bytes);
+    m.off = take(b, m.bytes);
     if (m.off == SIZE_MAX) return bfail(b, FHP_ENOMEM, "batch arena full: a %d x %d lattice needs %zu bytes", width, height, m.bytes);
     const size_t pb = fhp::round256(g.plane_words * sizeof(uint32_t));
     uint8_t* base = b->arena_base + m.off;
@@ -709,6 +730,7 @@ int fhp_batch_add(fhp_batch* b, int32_t width, int32_t height, uint64_t seed, do
     m.solid = (uint32_t*)(base + 14 * pb);
     m.flags = (unsigned int*)(base + 15 * pb);
     m.R = rows_per_tile(g, b->cur_quads);
+    for (int k : {2, 3}) m.lay[k - 2] = fhp::march_layout(g, k);
     cudaError_t e = cudaMemsetAsync(base, 0, m.bytes - kCanaryBytes, b->stream);
     if (e == cudaSuccess && kCanaryBytes)
         e = cudaMemsetAsync(base + m.bytes - kCanaryBytes, kCanaryByte, kCanaryBytes, b->stream);
@@ -1220,6 +1242,7 @@ void collect_trial(fhp_batch* b) {
     b->tuned[tr.cls] = best >= 0 ? tr.kind[best] : FHP_BATCH_KERNEL_SINGLE_STEP;
     b->tuned_quads[tr.cls] = best >= 0 ? tr.quads[best] : kDefaultTileQuads;
     b->tuned_block[tr.cls] = best >= 0 ? tr.block[best] : 1;
+    b->tuned_march[tr.cls] = best >= 0 && tr.march[best];
     tr.cls = -1;
 }
 
@@ -1253,7 +1276,7 @@ int run_chunk(fhp_batch* b, int chunk, int kind, std::vector<int>& steps_of, dou
 int ensure_block_tables(fhp_batch* b, size_t nm, size_t ntiles) {
     if (nm > b->bmem_cap) {
         const size_t cap = std::max<size_t>(nm, 2 * b->bmem_cap + 16);
-        const size_t off = b->arena.allocate(cap * sizeof(fhp::BlockMember));
+        const size_t off = take(b, cap * sizeof(fhp::BlockMember));
         if (off == SIZE_MAX) return bfail(b, FHP_ENOMEM, "batch arena full (blocked-pass descriptors)");
         if (b->bmem_off != SIZE_MAX) b->arena.release(b->bmem_off, b->bmem_cap * sizeof(fhp::BlockMember));
         b->bmem_off = off;
@@ -1262,7 +1285,7 @@ int ensure_block_tables(fhp_batch* b, size_t nm, size_t ntiles) {
     }
     if (ntiles > b->btile_cap) {
         const size_t cap = std::max<size_t>(ntiles, 2 * b->btile_cap + 256);
-        const size_t off = b->arena.allocate(cap * sizeof(fhp::BlockTile));
+        const size_t off = take(b, cap * sizeof(fhp::BlockTile));
         if (off == SIZE_MAX) return bfail(b, FHP_ENOMEM, "batch arena full (blocked-pass tile list)");
         if (b->btile_off != SIZE_MAX) b->arena.release(b->btile_off, b->btile_cap * sizeof(fhp::BlockTile));
         b->btile_off = off;
@@ -1371,6 +1394,190 @@ int run_blocked_chunk(fhp_batch* b, int chunk, int k, int kind, std::vector<int>
     return FHP_OK;
 }
 
+// Register marching: pass counters from the arena and the host's member
+// table.  False, leaving the batch's error message as it was, if the arena has
+// no room: the batch then does without.
+bool reserve_march(fhp_batch* b) {
+    if (b->d_march_flags) return true;
+    const size_t off = b->arena.allocate(kMarchFlagBytes);
+    if (off == SIZE_MAX) return false;
+    if (cudaMemsetAsync(b->arena_base + off, 0, kMarchFlagBytes, b->stream) != cudaSuccess) {
+        cudaGetLastError();
+        b->arena.release(off, kMarchFlagBytes);
+        return false;
+    }
+    b->march_epoch = 0;
+    b->d_march_flags = (unsigned int*)(b->arena_base + off);
+    if (b->h_march.empty()) b->h_march.resize(1);
+    return true;
+}
+
+// Members that march: enough rows, and forced nodes rare enough (p < 0.01) that
+// the walks do not outweigh the passes saved (64 lattices of 128 .. 2048 nodes a
+// side, GSUPS, marching against single steps: no forcing 4600 against 2900,
+// p = 5e-4 3470 against 2830, p = 0.02 2630 against 2720).
+bool marches(const Member& m, int k) {
+    return m.used && fhp::march_supported(m.g, k) && m.ft.p_plus_1 <= (1ull << 32) / 100;
+}
+
+// Steps per pass: 3 without forcing, except for batches whose bands would be
+// too low for a third level (see fhp::march_choice); 0 if no member marches.
+int march_block(const fhp_batch* b) {
+    long long nodes = 0;
+    bool force = false;
+    for (const Member& m : b->members) {
+        if (!marches(m, 2)) continue;
+        nodes += (long long)m.g.W * m.g.H;
+        force = force || m.ft.q[32] != 0;
+    }
+    if (nodes == 0) return 0;
+    return force || (nodes >= 24000000 && nodes < 48000000) ? 2 : 3;
+}
+
+// One cooperative launch per group of members: member i advances by
+// passes[i] passes of k steps.
+int launch_march_passes(fhp_batch* b, int k, const std::vector<int>& passes) {
+    const size_t nm = b->members.size();
+    bool force = false, ragged = false;
+    for (size_t i = 0; i < nm; ++i)
+        if (passes[i] > 0) {
+            force = force || b->members[i].ft.q[32] != 0;
+            ragged = ragged || b->members[i].g.Wq % 4 != 0;
+        }
+    int most = 0;
+    cudaError_t e = fhp::batch_march_ctas(k, force, ragged, &most);
+    if (e != cudaSuccess) return bcuda(b, e, "configuring the register-marching batch kernel");
+    auto ctas_for = [&](const Member& m, int R) {
+        return (int)((fhp::march_warps(m.g, m.lay[k - 2], R) + fhp::kMarchCtaWarps - 1) / fhp::kMarchCtaWarps);
+    };
+    size_t next = 0;
+    while (next < nm) {
+        // The next group: at most kMarchJobs members, which fit with bands as
+        // tall as they are.
+        std::vector<size_t> group;
+        int least = 0;
+        for (; next < nm && (int)group.size() < fhp::kMarchJobs; ++next)
+            if (passes[next] > 0) {
+                const int c = ctas_for(b->members[next], b->members[next].g.H);
+                if (least + c > most) break;
+                least += c;
+                group.push_back(next);
+            }
+        if (group.empty()) break;
+        // The lowest bands for which one resident wave of CTAs holds the group;
+        // beside forced members, whose walks cost about a third more time per
+        // row, the others get taller bands so that all end together.
+        std::vector<int> rows(group.size()), ctas(group.size());
+        int tallest = 0;
+        for (size_t i : group) tallest = std::max(tallest, b->members[i].g.H);
+        int total = 0;
+        for (int R = 2;; R += R < 16 ? 2 : (R / 8) & ~1) {
+            total = 0;
+            for (size_t j = 0; j < group.size(); ++j) {
+                const Member& m = b->members[group[j]];
+                rows[j] = fhp::march_rows(m.g, k, force && m.ft.q[32] == 0 ? (R + R / 3 + 1) & ~1 : R);
+                ctas[j] = ctas_for(m, rows[j]);
+                total += ctas[j];
+                if (total > most) break;
+            }
+            if (total <= most || R >= tallest) break;
+        }
+        if (total > most)
+            return bfail(b, FHP_ECUDA, "register marching: %zu members need %d CTAs of %d", group.size(), total, most);
+        fhp::MarchBatch& t = b->h_march[0];
+        t.flags = b->d_march_flags;
+        t.err = b->d_err;
+        // The counters are not cleared between launches: a launch's passes
+        // count on from where the counters can be (and once in 2^31 passes
+        // they start again).
+        int longest = 0;
+        for (size_t i : group) longest = std::max(longest, passes[i]);
+        if (b->march_epoch > 0x7FFFFFFFu - (unsigned int)longest) {
+            e = cudaMemsetAsync(b->d_march_flags, 0, kMarchFlagBytes, b->stream);
+            if (e != cudaSuccess) return bcuda(b, e, "clearing the pass counters");
+            b->march_epoch = 0;
+        }
+        t.epoch = b->march_epoch;
+        b->march_epoch += (unsigned int)longest;
+        int cta = 0;
+        for (size_t j = 0; j < group.size(); ++j) {
+            const Member& m = b->members[group[j]];
+            fhp::MarchJob& J = t.job[j];
+            J.src = m.buf[m.cur];
+            J.dst = m.buf[m.cur ^ 1];
+            J.solid = m.solid;
+            J.t0 = (unsigned long long)m.t;
+            J.P = m.ft.q[32] != 0 ? m.ft.p_plus_1 - 1 : 0;
+            J.plane_words = (uint32_t)m.g.plane_words;
+            J.H = m.g.H;
+            J.Wq = m.g.Wq;
+            J.key = fhp::Key2{(uint32_t)m.seed, (uint32_t)(m.seed >> 32)};
+            J.rest_rules = fhp::rest_rules_mask(m.g);
+            J.pre = m.ft.pre;
+            J.dense = m.ft.dense;
+            J.inv = m.ft.inv;
+            J.lay = m.lay[k - 2];
+            J.R = rows[j];
+            J.nbands = (m.g.H + rows[j] - 1) / rows[j];
+            J.nwarps = (int)fhp::march_warps(m.g, J.lay, rows[j]);
+            J.passes = passes[group[j]];
+            J.first_cta = cta;
+            for (int c = 0; c < ctas[j]; ++c) t.member[cta++] = (uint8_t)j;
+        }
+        e = fhp::launch_batch_march(t, cta, k, force, ragged, b->stream);
+        if (e != cudaSuccess) return bcuda(b, e, "launching the register-marching batch kernel");
+        ++b->launches;
+        for (size_t i : group) {
+            Member& m = b->members[i];
+            const int64_t adv = (int64_t)passes[i] * k;
+            m.t += adv;
+            m.cur ^= passes[i] & 1;
+            if (m.steps_left >= 0) m.steps_left -= adv;
+        }
+    }
+    return FHP_OK;
+}
+
+// One chunk by register marching: the members that march advance by passes of
+// k steps (k = 3: the remainder by up to two passes of 2), the steps left over
+// (all steps of the other members) run on the batch step kernel `kind`.  The
+// result equals single steps for every member.
+int run_march_chunk(fhp_batch* b, int chunk, int k, int kind, std::vector<int>& steps_of, double* updates) {
+    const size_t nm = b->members.size();
+    if (!reserve_march(b)) return run_chunk(b, chunk, kind, steps_of, updates);
+    std::vector<int> left(nm, 0), passes(nm, 0);
+    steps_of.assign(nm, 0);
+    double upd = 0.0;
+    for (size_t i = 0; i < nm; ++i) {
+        const Member& m = b->members[i];
+        if (!m.used) continue;
+        int64_t s = chunk;
+        if (m.steps_left >= 0 && m.steps_left < s) s = m.steps_left;
+        left[i] = steps_of[i] = (int)s;
+        upd += (double)m.g.W * m.g.H * (double)s;
+    }
+    for (; k >= 2; --k) {
+        bool any = false;
+        for (size_t i = 0; i < nm; ++i) {
+            passes[i] = 0;
+            if (left[i] < 2 || !marches(b->members[i], k)) continue;
+            // k = 3: what remains is even (1 step is 2 + 2 less a pass of 3).
+            passes[i] = k == 2 ? left[i] / 2 : left[i] % 3 == 1 ? (left[i] - 4) / 3 : left[i] / 3;
+            if (passes[i] < 0) passes[i] = 0;
+            left[i] -= passes[i] * k;
+            any = any || passes[i] > 0;
+        }
+        if (!any) continue;
+        const int rc = launch_march_passes(b, k, passes);
+        if (rc != FHP_OK) return rc;
+    }
+    std::vector<int> rest_of;
+    const int rc = run_chunk(b, chunk, kind, rest_of, nullptr, &left);
+    if (rc != FHP_OK) return rc;
+    if (updates) *updates = upd;
+    return FHP_OK;
+}
+
 }  // namespace
 
 namespace {
@@ -1415,6 +1622,7 @@ int batch_step(fhp_batch* b, int64_t n) {
                 tr.kind[nc] = kind;
                 tr.quads[nc] = b->tile_quads ? b->tile_quads : sizes[si];
                 tr.block[nc] = b->temporal_block > 1 ? b->temporal_block : 1;
+                tr.march[nc] = false;
                 ++nc;
             }
         const int64_t min_part = std::max<int64_t>(kTuneMinSteps, b->graph_steps);
@@ -1426,13 +1634,16 @@ int batch_step(fhp_batch* b, int64_t n) {
                 // trial goes on with the others.
                 if (n >= (nc + 2) * min_part) {
                     trial = true;
-                    if (reserve_block_tables(b))
-                        for (int k : {2, 4}) {
-                            tr.kind[nc] = FHP_BATCH_KERNEL_SINGLE_STEP;
-                            tr.quads[nc] = b->tile_quads ? b->tile_quads : kDefaultTileQuads;
-                            tr.block[nc] = k;
-                            ++nc;
-                        }
+                    const bool blocked = reserve_block_tables(b);
+                    const int mk = reserve_march(b) ? march_block(b) : 0;
+                    for (int k : {mk ? mk : (blocked ? 2 : 0), blocked ? 4 : 0}) {
+                        if (k == 0) continue;
+                        tr.kind[nc] = FHP_BATCH_KERNEL_SINGLE_STEP;
+                        tr.quads[nc] = b->tile_quads ? b->tile_quads : kDefaultTileQuads;
+                        tr.block[nc] = k;
+                        tr.march[nc] = k != 4 && mk != 0;
+                        ++nc;
+                    }
                 }
             } else {
                 trial = n >= nc * min_part;
@@ -1471,8 +1682,9 @@ int batch_step(fhp_batch* b, int64_t n) {
                 if (rc != FHP_OK) return rc;
                 cudaEventRecord(tr.ev[k][0], b->stream);
                 tr.updates[k] = 0.0;
-                rc = tr.block[k] > 1 ? run_blocked_chunk(b, part, tr.block[k], tr.kind[k], steps_of, &tr.updates[k])
-                                     : run_chunk(b, part, tr.kind[k], steps_of, &tr.updates[k]);
+                rc = tr.march[k]   ? run_march_chunk(b, part, tr.block[k], tr.kind[k], steps_of, &tr.updates[k])
+                     : tr.block[k] > 1 ? run_blocked_chunk(b, part, tr.block[k], tr.kind[k], steps_of, &tr.updates[k])
+                                       : run_chunk(b, part, tr.kind[k], steps_of, &tr.updates[k]);
                 if (rc != FHP_OK) return rc;
                 cudaError_t e = cudaEventRecord(tr.ev[k][1], b->stream);
                 if (e != cudaSuccess) return bcuda(b, e, "recording the tuning events");
@@ -1501,10 +1713,23 @@ int batch_step(fhp_batch* b, int64_t n) {
             kind = t == FHP_BATCH_KERNEL_AUTO ? FHP_BATCH_KERNEL_SINGLE_STEP : t;
         }
         // Temporal block: the caller's, else (with the automatic kernel) the
-        // one recorded for the class, else none.
+        // one recorded for the class, else register marching.
         int k = b->temporal_block;
-        if (k == 0) k = (b->step_kernel == FHP_BATCH_KERNEL_AUTO && b->tuned_block[cls]) ? b->tuned_block[cls] : 1;
-        rc = k > 1 ? run_blocked_chunk(b, chunk, k, kind, steps_of, nullptr) : run_chunk(b, chunk, kind, steps_of, nullptr);
+        bool march = false;
+        if (k == 0 && b->step_kernel == FHP_BATCH_KERNEL_AUTO) {
+            if (b->tuned_block[cls]) {
+                k = b->tuned_block[cls];
+                march = b->tuned_march[cls];
+            } else {
+                march = chunk >= 2 && reserve_march(b);
+            }
+            if (march) k = march_block(b);   // (the members may have changed since the trial)
+            march = march && k != 0;
+        }
+        if (k == 0) k = 1;
+        rc = march   ? run_march_chunk(b, chunk, k, kind, steps_of, nullptr)
+             : k > 1 ? run_blocked_chunk(b, chunk, k, kind, steps_of, nullptr)
+                     : run_chunk(b, chunk, kind, steps_of, nullptr);
         if (rc != FHP_OK) return rc;
         left -= chunk;
     }

@@ -186,6 +186,52 @@ cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const 
                          bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int k, int passes,
                          unsigned int* flags, size_t flag_bytes, cudaStream_t stream, unsigned int* err);
 
+struct MarchLayout {
+    int pitch;      // chain positions per band (0: whole rows in a warp)
+    int left;       // chain positions left of a band's quad 0
+    int hl;         // halo lanes per side of a warp (chain)
+    int per_warp;   // whole rows: bands per warp
+};
+MarchLayout march_layout(const Geometry& g, int k);
+long long march_warps(const Geometry& g, const MarchLayout& l, int R);   // warps for bands of R rows
+int march_rows(const Geometry& g, int k, int R);                         // band height allowed from R on
+
+// Register marching of a batch (fhp_batch_march.cu): all passes of k (2 or 3)
+// steps of up to kMarchJobs members in one cooperative launch.  The member
+// table is a kernel parameter, and a CTA (kMarchCtaWarps warps) works for one
+// member, so that its fields are uniform operands as in the single-lattice
+// kernel (read from device memory into registers they spilled: 88 to 560 bytes
+// a thread).
+constexpr int kMarchJobs = 256;
+constexpr int kMarchMaxCtas = 640;
+constexpr int kMarchCtaWarps = 4;
+struct MarchJob {
+    uint32_t* src;             // state at t0; the result where `passes` is even
+    uint32_t* dst;
+    const uint32_t* solid;
+    unsigned long long t0;
+    unsigned long long P;      // round(p * 2^32)
+    uint32_t plane_words;
+    int H, Wq;
+    Key2 key;
+    uint32_t rest_rules;
+    uint32_t pre, dense, inv;  // forcing (ForcingTable)
+    MarchLayout lay;
+    int R, nbands, nwarps, passes;
+    int first_cta;             // the member's first CTA
+};
+struct MarchBatch {
+    MarchJob job[kMarchJobs];
+    uint8_t member[kMarchMaxCtas];   // CTA -> job
+    unsigned int* flags;             // kMarchCtaWarps words per CTA: passes finished, counted from `epoch`
+    unsigned int* err;
+    unsigned int epoch;              // no word is above this at launch
+};
+static_assert(sizeof(MarchBatch) <= 32764, "kernel parameters are limited to 32,764 bytes");
+// CTAs one launch may have (all must be resident; at most kMarchMaxCtas).
+cudaError_t batch_march_ctas(int k, bool force, bool ragged, int* ctas);
+cudaError_t launch_batch_march(const MarchBatch& t, int ctas, int k, bool force, bool ragged, cudaStream_t stream);
+
 // Pack H x W node bytes (device) into 7 state planes + the solid plane.
 // Sets *device_any_solid to a nonzero value if any node is solid.
 cudaError_t launch_pack(const Geometry& g, const uint8_t* bytes, uint32_t* state,

@@ -19,45 +19,63 @@ int march_sms() {
     return sms[dev];
 }
 
-// True if every useful lane of the chain keeps k valid words on both sides:
-// a level spoils one more word inwards from each end of a warp, and a partial
-// last quad has only m words to spare.
-bool chain_valid(int nq, int m, int k, int pitch, int left, int hl) {
-    if (m >= k) return true;
-    const int step = 32 - 2 * hl;
-    // Warps start at chain positions 0, step, 2 step, ...; the positions
-    // modulo the pitch repeat after at most `pitch` warps.
-    for (int w = 0, start = 0; w < pitch; ++w, start = (start + step) % pitch) {
-        for (int lane = hl; lane < 32 - hl; ++lane) {
-            const int e = (start + lane) % pitch, q = e - left;
-            if (q < 0 || q >= nq) continue;
-            int words = 0;
-            for (int l = lane - 1; l >= 0 && words < k; --l) {
-                const int qq = ((q - (lane - l)) % nq + nq) % nq;
-                words += qq == nq - 1 ? m : 4;
-            }
-            if (words < k) return false;
-            words = 0;
-            for (int l = lane + 1; l <= 31 && words < k; ++l) {
-                const int qq = (q + (l - lane)) % nq;
-                words += qq == nq - 1 ? m : 4;
-            }
-            if (words < k) return false;
-        }
-    }
-    return true;
-}
-
-}  // namespace
-
-namespace {
-
 cudaError_t march_any(int k, const StepArgs& a, const MarchArgs& b, const MarchVariant& v, bool launch, int* n,
                       cudaStream_t s) {
     return k == 2 ? march_k<2>(a, b, v, launch, n, s) : march_k<3>(a, b, v, launch, n, s);
 }
 
 }  // namespace
+
+// How the quad columns of a lattice's bands go to lanes.  Rows of few quads:
+// whole rows side by side in a warp (periodic in x by the shuffles' source
+// lanes) where that fills the warp at least as well as the chain.  Else one
+// chain of all bands' columns, each band with its halo columns, cut every 30
+// lanes: about 92 % of the lanes for rows of 128 quads.
+//
+// A level spoils one more word inwards from each end of what a warp holds of
+// a band, so a halo quad must hold k words.  All do but a partial last quad of
+// m < k words.  Then a band has two halo columns to its left, and no warp may
+// begin at the second of them or end at the last column: warps begin at the
+// multiples of g = gcd(30, pitch) modulo the pitch, so g > 1 must not divide the
+// number of quads.  The pitch is raised to the next one with that property, or
+// the warps get two halo lanes per side (28 columns) where that is cheaper.
+MarchLayout march_layout(const Geometry& g, int k) {
+    MarchLayout l{};
+    const int m = g.Wq - 4 * (g.nq - 1);
+    const int whole = g.nq <= 32 ? 32 / g.nq : 0;
+    if (whole && whole * (g.nq + 2) >= 30) {
+        l.per_warp = whole;
+        return l;
+    }
+    l.hl = 1;
+    l.left = 1;
+    l.pitch = g.nq + 2;
+    if (m >= k) return l;
+    l.left = 2;
+    auto gcd30 = [](int v) { return (v % 2 ? 1 : 2) * (v % 3 ? 1 : 3) * (v % 5 ? 1 : 5); };
+    for (l.pitch = g.nq + 3; l.pitch * 28 <= (g.nq + 4) * 30; ++l.pitch) {
+        const int d = gcd30(l.pitch);
+        if (d > 1 && g.nq % d != 0) return l;
+    }
+    l.hl = 2;
+    l.pitch = g.nq + 4;
+    return l;
+}
+
+long long march_warps(const Geometry& g, const MarchLayout& l, int R) {
+    const long long bands = (g.H + R - 1) / R;
+    if (!l.pitch) return (bands + l.per_warp - 1) / l.per_warp;
+    const int step = 32 - 2 * l.hl;
+    return (bands * l.pitch + step - 1) / step;
+}
+
+// (Every band, the last one too, has at least k rows, so that a pass reads no
+// further than the next band.)
+int march_rows(const Geometry& g, int k, int R) {
+    if (R < k) R = (k + 1) & ~1;
+    while (R < g.H && g.H % R != 0 && g.H % R < k) R += 2;
+    return R < g.H ? R : g.H;
+}
 
 bool march_supported(const Geometry& g, int k) {
     return (k == 2 || k == 3) && g.H >= 2 * k + 2 && g.plane_words * 4 < ((size_t)1 << 32) - 64;
@@ -114,50 +132,18 @@ cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const 
     const int resident = march_sms() * per_sm * kMarchWarps;
     if (resident <= 0) return cudaErrorInvalidDevice;
 
-    // How a band's columns go to lanes: whole rows side by side in a warp
-    // (periodic in x by the shuffles' source lanes) where that fills the warp
-    // at least as well, else one chain of all bands' columns, each band with
-    // its halo columns, cut every 30 lanes (28 where a partial last quad is
-    // too narrow to be a halo): about 92 % of the lanes for rows of 128 quads.
-    const int m = g.Wq - 4 * (g.nq - 1);
-    const int whole = g.nq <= 32 ? 32 / g.nq : 0;
-    if (whole && whole * g.nq * (g.nq + 2) >= 30 * g.nq) {
-        b.per_warp = whole;
-    } else {
-        b.hl = 1;
-        b.left = 1;
-        b.pitch = g.nq + 2;
-        if (!chain_valid(g.nq, m, k, b.pitch, 1, 1)) {
-            int best = 0;
-            for (int left = 1; left <= 2; ++left)
-                for (int pad = left + 1; pad < 32 && (!best || g.nq + pad < best); ++pad)
-                    if (chain_valid(g.nq, m, k, g.nq + pad, left, 1)) {
-                        best = g.nq + pad;
-                        b.left = left;
-                    }
-            b.pitch = best;
-            if (!best || best * 28 > (g.nq + 4) * 30) {   // two halo lanes always hold k words
-                b.hl = 2;
-                b.left = 2;
-                b.pitch = g.nq + 4;
-            }
-        }
-    }
-    const int step = 32 - 2 * b.hl;
-    auto warps_for = [&](int r) -> long long {
-        const long long nb = (g.H + r - 1) / r;
-        return b.pitch ? (nb * b.pitch + step - 1) / step : (nb + b.per_warp - 1) / b.per_warp;
-    };
-    // The lowest bands that one resident wave of warps covers.  Every band,
-    // the last one too, has at least k rows, so that a pass reads no further
-    // than the next band.
-    int R = k <= 2 ? 2 : 4;
-    while (R < g.H && (warps_for(R) > resident || (g.H % R != 0 && g.H % R < k))) R += 2;
-    if (R > g.H) R = g.H;
-    if (warps_for(R) > resident) return cudaErrorInvalidConfiguration;
+    const MarchLayout lay = march_layout(g, k);
+    b.pitch = lay.pitch;
+    b.left = lay.left;
+    b.hl = lay.hl;
+    b.per_warp = lay.per_warp;
+    // The lowest bands that one resident wave of warps covers.
+    int R = march_rows(g, k, 2);
+    while (R < g.H && march_warps(g, lay, R) > resident) R = march_rows(g, k, R + 2);
+    if (march_warps(g, lay, R) > resident) return cudaErrorInvalidConfiguration;
     b.R = R;
     b.nbands = (g.H + R - 1) / R;
-    b.nwarps = (int)warps_for(R);
+    b.nwarps = (int)march_warps(g, lay, R);
     b.flags = flags;
     const size_t need = (size_t)b.nwarps * sizeof(unsigned int);
     const int per_launch = need <= flag_bytes ? passes : 1;

@@ -33,7 +33,8 @@ struct MarchArgs {
     int per_warp;   // whole rows: bands per warp
     int nwarps;
     int passes;     // passes of k steps in the launch
-    unsigned int* flags;   // passes > 1: per warp, passes finished (zero at launch)
+    unsigned int* flags;   // passes > 1: per warp, passes finished, counted from `epoch`
+    unsigned int epoch;    // no flag is above this at launch
 };
 
 constexpr int kMarchWarps = 4;   // warps per CTA (independent of one another)
@@ -282,7 +283,8 @@ __device__ __noinline__ bool march_wait(const unsigned int* flags, int neighbour
 }
 
 template <int K, bool SOLID, bool FORCE, bool RAGGED, bool SAT>
-__device__ __forceinline__ void march_warp(const StepArgs& a, const MarchArgs& b, int gw, uint32_t ring) {
+__device__ __forceinline__ void march_warp(const StepArgs& a, const MarchArgs& b, int gw, uint32_t ring,
+                                           uint32_t q_lane) {
     using Ring = MarchRing<K, SOLID>;
     constexpr int D = Ring::stages;
     const int lane = (int)threadIdx.x & 31;
@@ -294,7 +296,6 @@ __device__ __forceinline__ void march_warp(const StepArgs& a, const MarchArgs& b
     const uint32_t solid_base = lane_base + (uint32_t)(D * 7 * 512);
     const size_t pb = (size_t)a.plane_words * 4;
     const int ticks = b.R + 2 * (K - 1);
-    const uint32_t q_lane = FORCE ? (uint32_t)(a.ft.q[lane + 1] - 1ull) : 0u;
     int neighbour = -1;
     if (b.passes > 1) 
         neighbour = march_neighbours(a.nq, b.nbands, b.pitch, b.left, b.hl, b.per_warp, L.y0 / b.R, L.q, lane);
@@ -303,7 +304,7 @@ __device__ __forceinline__ void march_warp(const StepArgs& a, const MarchArgs& b
     for (int pass = 0; pass < b.passes; ++pass) {
     const char* src = reinterpret_cast<const char*>((pass & 1) ? a.dst : a.src);
     char* dst = reinterpret_cast<char*>((pass & 1) ? const_cast<uint32_t*>(a.src) : a.dst);
-    if (pass > 0 && !march_wait(b.flags, neighbour, (unsigned int)pass)) {
+    if (pass > 0 && !march_wait(b.flags, neighbour, b.epoch + (unsigned int)pass)) {
         if (lane == 0 && a.err) atomicOr(a.err, 1u);
         return;
     }
@@ -478,7 +479,8 @@ __device__ __forceinline__ void march_warp(const StepArgs& a, const MarchArgs& b
         __syncwarp();
         if (lane == 0) {
             asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(b.flags + gw), "r"(pass + 1) : "memory");
+            asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(b.flags + gw), "r"(b.epoch + (unsigned int)pass + 1u)
+                         : "memory");
         }
     }
     }
@@ -492,7 +494,8 @@ __global__ void __launch_bounds__(32 * kMarchWarps, K <= 2 ? 4 : (K == 3 ? 3 : 2
     const int gw = (int)blockIdx.x * kMarchWarps + warp;
     if (gw >= b.nwarps) return;
     march_warp<K, SOLID, FORCE, RAGGED, SAT>(
-        a, b, gw, smem_addr(smem_raw) + (uint32_t)(warp * MarchRing<K, SOLID>::warp_bytes));
+        a, b, gw, smem_addr(smem_raw) + (uint32_t)(warp * MarchRing<K, SOLID>::warp_bytes),
+        FORCE ? (uint32_t)(a.ft.q[(threadIdx.x & 31) + 1] - 1ull) : 0u);
 }
 
 template <int K, bool SOLID, bool FORCE, bool RAGGED, bool SAT>

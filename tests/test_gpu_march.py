@@ -66,7 +66,7 @@ def test_march_every_candidate_forced_and_full(pkg, oracle_mod):
         assert np.array_equal(got, want)
 
 
-@pytest.mark.parametrize("W,H,p,block", [(4096, 4096, 0.0, 3), (8192, 4096, 0.0, 2), (16384, 2560, 5e-4, 2),
+@pytest.mark.parametrize("W,H,p,block", [(8192, 2560, 0.0, 3), (8192, 4096, 0.0, 2), (16384, 2560, 5e-4, 2),
                                          (12032, 3400, 1e-3, 2)])
 def test_automatic_choice_equals_direct_kernel(pkg, W, H, p, block):
     import torch
@@ -90,3 +90,51 @@ def test_march_refusals(pkg):
             with pytest.raises(pkg.FhpError):
                 lat.step_march(k, n)
         assert lat.t == 0
+
+
+def test_batch_members_march(pkg, oracle_mod):
+    """A batch with automatic settings marches the members that can (any row
+    width, rare forcing) and steps the others (two rows, dense forcing) singly:
+    every member equals its oracle run over calls of 1 to 67 steps and with
+    step budgets, with and without forced members (passes of 2 and of 3)."""
+    rng = np.random.Generator(np.random.PCG64(3))
+    sizes = [(32, 8), (96, 40), (128, 128), (320, 200), (1056, 66), (2048, 30), (4128, 26), (8224, 14), (256, 2), (640, 4)]
+    for forced in (False, True):
+        jobs = [workloads.Lattice(f"m{i}", W, H, float(rng.uniform(0.1, 0.5)), 700 + i,
+                                  {1: 0.01, 4: 0.001, 3: 0.3}.get(i, 0.0) if forced else 0.0, 0,
+                                  obstacle="points" if i % 2 else "none", point_frac=0.02)
+                for i, (W, H) in enumerate(sizes)]
+        states = [j.initial_state() for j in jobs]
+        with pkg.Batch(sum(pkg.Batch.lattice_bytes(j.W, j.H) for j in jobs) + (64 << 20)) as b:
+            slots = []
+            for j, s0 in zip(jobs, states):
+                k = b.add(j.W, j.H, j.seed, j.p)
+                b.set_state(k, s0)
+                b.set_time(k, 2**32 - 9)
+                slots.append(k)
+            b.set_rules(slots[2], 1)
+            b.set_steps_left(slots[5], 11)
+            for n in (2, 3, 4, 5, 67, 1):
+                b.step(n)
+            b.synchronize()
+            for i, (j, s0, k) in enumerate(zip(jobs, states, slots)):
+                n = 11 if i == 5 else 82
+                want, _ = oracle_mod.run(s0, j.seed, 2**32 - 9, n, j.p, rules=1 if i == 2 else 2)
+                assert b.time(k) == 2**32 - 9 + n
+                assert np.array_equal(b.get_state(k), want), (j.W, j.H, forced)
+
+
+def test_batch_of_more_members_than_a_launch_holds(pkg, oracle_mod):
+    """300 members: more than one group of 256; a wide one among them."""
+    jobs = [(64, 16, 900 + i, 0.3) for i in range(299)] + [(8192, 64, 1300, 0.2)]
+    with pkg.Batch(sum(pkg.Batch.lattice_bytes(w, h) for w, h, *_ in jobs) + (32 << 20)) as b:
+        slots = []
+        for w, h, seed, rho in jobs:
+            k = b.add(w, h, seed, 0.0)
+            b.init_random(k, rho)
+            slots.append(k)
+        b.step(6)
+        for i in (0, 255, 256, 298, 299):
+            w, h, seed, rho = jobs[i]
+            want, _ = oracle_mod.run(oracle_mod.init_random(w, h, seed, rho), seed, 0, 6, 0.0)
+            assert np.array_equal(b.get_state(slots[i]), want), i
