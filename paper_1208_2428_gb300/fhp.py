@@ -496,26 +496,33 @@ class Batch:
         s = self._side
         H, W = self.shapes[slot]
         nby, nbx = H // block, W // block
+        # counts, rho, ux, uy back to back: one device buffer, one pinned
+        # buffer and one copy (an allocation and a copy per field cost 75 us of
+        # host time a call, more than the copies themselves).
+        cells = nby * nbx
         if after_event is not None:
             s.wait_event(after_event)
         with torch.cuda.stream(s):
-            dev = [torch.empty((nby, nbx, 9), dtype=torch.int32, device=self.device)] + \
-                  [torch.empty((nby, nbx), dtype=torch.float32, device=self.device) for _ in range(3)]
+            dev = torch.empty(cells * 48, dtype=torch.uint8, device=self.device)
+            p = dev.data_ptr()
             self._check(self._lib.fhp_batch_coarse_grain_device(
-                self._h, int(slot), int(block), *[ctypes.c_void_p(t.data_ptr()) for t in dev],
-                ctypes.c_void_p(s.cuda_stream)))
-            host = [torch.empty(t.shape, dtype=t.dtype, pin_memory=True) for t in dev]
-            for hsrc, dsrc in zip(host, dev):
-                hsrc.copy_(dsrc, non_blocking=True)
-        return (s, dev, host)
+                self._h, int(slot), int(block), ctypes.c_void_p(p), ctypes.c_void_p(p + cells * 36),
+                ctypes.c_void_p(p + cells * 40), ctypes.c_void_p(p + cells * 44), ctypes.c_void_p(s.cuda_stream)))
+            host = torch.empty(cells * 48, dtype=torch.uint8, pin_memory=True)
+            host.copy_(dev, non_blocking=True)
+        return (s, dev, host, (nby, nbx))
 
     @staticmethod
     def coarse_grain_finish(handle):
         """Wait for a read-back started by coarse_grain_begin; returns
         (counts, rho, ux, uy) as numpy arrays."""
-        s, dev, host = handle
+        s, dev, host, (nby, nbx) = handle
         s.synchronize()
-        return tuple(h.numpy() for h in host)
+        h = host.numpy()
+        cells = nby * nbx
+        counts = h[:cells * 36].view(np.int32).reshape(nby, nbx, 9)
+        return (counts,) + tuple(h[cells * (36 + 4 * i):cells * (40 + 4 * i)].view(np.float32).reshape(nby, nbx)
+                                 for i in range(3))
 
     def set_state(self, slot: int, state: np.ndarray):
         s = np.ascontiguousarray(state, dtype=np.uint8)
