@@ -202,8 +202,9 @@ FHP_API int fhp_load_obstacle_shapes(fhp_lattice* lattice, const fhp_shape* shap
  * swap, and the three-state classes of momentum c_k cycle (chirality sets the
  * direction); it keeps every FHP-II collision.  FHP-III lattices step with
  * the direct, bulk-copy ring and multi-step ring kernels (step kernels 1-3;
- * the resident kernel and temporal blocks k > 1 fall back to those) and
- * cannot be batch members.  Takes effect from the next step.
+ * kernel 4 and temporal blocks k > 1 fall back to those; the automatic choice
+ * and kernel 4 keep a lattice that fits in shared memory for the steps of a
+ * call, reported as kernel 3) and cannot be batch members.  Takes effect from the next step.
  * FHP_EINVAL for other values. */
 #define FHP_RULES_FHP_I 1
 #define FHP_RULES_FHP_II 2
@@ -283,8 +284,8 @@ FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
  * running all steps of an fhp_step call in one cooperative launch, each tile
  * waiting only for the three tiles of the previous step it reads).  2 and 3
  * fall back to 1 when a row does not fit a stage.  Automatic picks 4 for
- * lattices whose strips fit (calls of up to three steps: 1; FHP-III lattices:
- * never 4), else register marching for lattices of 12 million nodes and more
+ * lattices whose strips fit (calls of up to three steps: 1; FHP-III lattices
+ * report it as 3, all steps of a call in one launch), else register marching for lattices of 12 million nodes and more
  * (40 million with forcing, whose probability must be below 0.0025; 200
  * million for forced FHP-III lattices): passes of 2 or 3 steps in which every
  * lane of a warp marches a column of 128-node quads up a band of rows with

@@ -190,6 +190,12 @@ void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk
     }
 }
 
+// The number under which a kernel is reported: an FHP-III lattice in shared
+// memory runs under that of the kernel that takes all steps in one launch.
+int reported_kernel(const fhp_lattice* h, int kernel) {
+    return h->g.rules == 3 && kernel == fhp::kStepResident ? fhp::kStepRun : kernel;
+}
+
 // Steps between exchanges of the resident kernel for these settings (2 when
 // asked for and supported, else 1), or 0 if the resident kernel does not run.
 int resident_interval(const fhp_lattice* h, int kernel, int k_block) {
@@ -673,7 +679,7 @@ int fhp_get_step_kernel(const fhp_lattice* h) {
     effective_settings(h, &kernel, &k_block);
     if (kernel == fhp::kStepResident)
         return fhp::resident_supported(h->g, h->has_solid, h->staging_bytes)
-                   ? fhp::kStepResident
+                   ? reported_kernel(h, kernel)
                    : fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepAuto);
     return fhp::resolved_step_kernel(h->g, h->has_solid, kernel);
 }
@@ -853,7 +859,7 @@ int fhp_autotune(fhp_lattice* h, int32_t trial_steps, int32_t* out_kernel, int32
     h->k_block = 1;
     h->block_kernel = 0;
     record_tuned(TuneKey{h->device, h->g.W, h->g.H, h->has_solid, h->force, h->g.rules}, best);
-    if (out_kernel) *out_kernel = best.kernel;
+    if (out_kernel) *out_kernel = reported_kernel(h, best.kernel);
     if (out_temporal_block) *out_temporal_block = best.k;
     return FHP_OK;
 }

@@ -79,7 +79,8 @@ __device__ __forceinline__ bool get_unit(const unsigned long long* unit, uint32_
     }
 }
 
-template <bool SOLID, bool FORCE, bool RAGGED>
+// SAT: the FHP-III rule set.
+template <bool SOLID, bool FORCE, bool RAGGED, bool SAT>
 __global__ void __launch_bounds__(kRes1Threads, 1) fhp_resident_kernel(const StepArgs a, const ResArgs ra) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int T = kRes1Threads;
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(kRes1Threads, 1) fhp_resident_kernel(const Ste
         };
         uint4 o[7];
         if (tid < items) {
-            resident_quad_drawn<SOLID, FORCE, RAGGED>(a, v, src, dst, S + (size_t)rr0 * Pq, pstride, rr0 + 1, y0 + rr0,
+            resident_quad_drawn<SOLID, FORCE, RAGGED, SAT>(a, v, src, dst, S + (size_t)rr0 * Pq, pstride, rr0 + 1, y0 + rr0,
                                                       q0, chi, gate, o);
             if (tid < edge) hand_over(rr0, q0, o);
             if (more) resident_draws<FORCE>(a, step_of(s + 1), q0, y0 + rr0, chi, gate);
@@ -177,7 +178,7 @@ __global__ void __launch_bounds__(kRes1Threads, 1) fhp_resident_kernel(const Ste
         for (int e = tid + T; e < items; e += T) {
             int rr, q;
             place(e, rr, q);
-            resident_quad_at<SOLID, FORCE, RAGGED>(a, v, src, dst, S + (size_t)rr * Pq, pstride, rr + 1, y0 + rr, q, o);
+            resident_quad_at<SOLID, FORCE, RAGGED, SAT>(a, v, src, dst, S + (size_t)rr * Pq, pstride, rr + 1, y0 + rr, q, o);
             if (e < edge) hand_over(rr, q, o);
         }
         if (G > 1 && more) {
@@ -211,30 +212,35 @@ __global__ void __launch_bounds__(kRes1Threads, 1) fhp_resident_kernel(const Ste
 
 std::mutex g_res_mutex;
 int g_res_sms[64] = {};
-bool g_res_configured[64][2][2][2] = {};
+bool g_res_configured[64][2][2][2][2] = {};
 
-template <bool SOLID, bool FORCE, bool RAGGED>
+template <bool SOLID, bool FORCE, bool RAGGED, bool SAT>
 cudaError_t launch_resident_variant(const StepArgs& a, const ResArgs& ra, int grid, size_t smem, cudaStream_t s) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    return launch_resident_coop((const void*)fhp_resident_kernel<SOLID, FORCE, RAGGED>,
-                                &g_res_configured[dev][SOLID][FORCE][RAGGED], a, ra, grid, kRes1Threads, smem, s);
+    return launch_resident_coop((const void*)fhp_resident_kernel<SOLID, FORCE, RAGGED, SAT>,
+                                &g_res_configured[dev][SOLID][FORCE][RAGGED][SAT], a, ra, grid, kRes1Threads, smem, s);
+}
+
+template <bool SOLID, bool FORCE>
+cudaError_t launch_resident_sf(const StepArgs& a, const ResArgs& ra, int grid, size_t smem, bool ragged, bool sat,
+                               cudaStream_t s) {
+    if (sat)
+        return ragged ? launch_resident_variant<SOLID, FORCE, true, true>(a, ra, grid, smem, s)
+                      : launch_resident_variant<SOLID, FORCE, false, true>(a, ra, grid, smem, s);
+    return ragged ? launch_resident_variant<SOLID, FORCE, true, false>(a, ra, grid, smem, s)
+                  : launch_resident_variant<SOLID, FORCE, false, false>(a, ra, grid, smem, s);
 }
 
 cudaError_t launch_resident_one(const StepArgs& a, const ResArgs& ra, int grid, size_t smem, bool has_solid,
-                                bool force, bool ragged, cudaStream_t s) {
-    if (has_solid) {
-        if (force) return ragged ? launch_resident_variant<true, true, true>(a, ra, grid, smem, s)
-                                 : launch_resident_variant<true, true, false>(a, ra, grid, smem, s);
-        return ragged ? launch_resident_variant<true, false, true>(a, ra, grid, smem, s)
-                      : launch_resident_variant<true, false, false>(a, ra, grid, smem, s);
-    }
-    if (force) return ragged ? launch_resident_variant<false, true, true>(a, ra, grid, smem, s)
-                             : launch_resident_variant<false, true, false>(a, ra, grid, smem, s);
-    return ragged ? launch_resident_variant<false, false, true>(a, ra, grid, smem, s)
-                  : launch_resident_variant<false, false, false>(a, ra, grid, smem, s);
+                                bool force, bool ragged, bool sat, cudaStream_t s) {
+    if (has_solid)
+        return force ? launch_resident_sf<true, true>(a, ra, grid, smem, ragged, sat, s)
+                     : launch_resident_sf<true, false>(a, ra, grid, smem, ragged, sat, s);
+    return force ? launch_resident_sf<false, true>(a, ra, grid, smem, ragged, sat, s)
+                 : launch_resident_sf<false, false>(a, ra, grid, smem, ragged, sat, s);
 }
 
 }  // namespace
@@ -297,7 +303,7 @@ size_t resident_halo_words(const Geometry& g, bool has_solid, int gh) {
 }
 
 bool resident_supported(const Geometry& g, bool has_solid, size_t staging_bytes, int gh) {
-    if ((gh != 1 && gh != 2) || g.rules == 3) return false;   // FHP-III: not in the resident kernels
+    if ((gh != 1 && gh != 2) || (gh > 1 && g.rules == 3)) return false;   // (two ghost rows: not FHP-III)
     const int grid = resident_grid(g, has_solid, gh);
     if (grid <= 0) return false;
     if (gh > 1 && g.H / grid < 2 * gh) return false;   // every strip holds its 2 gh edge rows
@@ -345,7 +351,7 @@ cudaError_t launch_resident(const Geometry& g, uint32_t* buf0, uint32_t* buf1, c
         e = cudaMemsetAsync(halo, 0, resident_halo_words(g, has_solid, 1) * sizeof(uint32_t), stream);
     if (e != cudaSuccess) return e;
     const bool ragged = g.Wq % 4 != 0;
-    return gh == 1 ? launch_resident_one(a, ra, grid, smem, has_solid, force, ragged, stream)
+    return gh == 1 ? launch_resident_one(a, ra, grid, smem, has_solid, force, ragged, g.rules == 3, stream)
                    : launch_resident_ghost2(a, ra, grid, smem, has_solid, force, ragged, stream);
 }
 

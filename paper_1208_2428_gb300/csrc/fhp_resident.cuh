@@ -74,7 +74,7 @@ __device__ __noinline__ bool wait_neighbours(const unsigned int* flags, int p, i
 // of the new state into `dst` (padding words of a ragged row stay zero).
 // (Local row lr of the staged buffers, lattice row y, `Srow` its solid row.)
 // (resident_quad_drawn takes the quad's random blocks from the caller.)
-template <bool SOLID, bool FORCE, bool RAGGED>
+template <bool SOLID, bool FORCE, bool RAGGED, bool SAT = false>
 __device__ __forceinline__ void resident_quad_drawn(const StepArgs& a, const StepVar& v, const uint32_t* src,
                                                     uint32_t* dst, const uint32_t* Srow, size_t pstride, int lr, int y,
                                                     int q, uint4 chi, uint4 gate, uint4 (&o)[7]) {
@@ -108,7 +108,7 @@ __device__ __forceinline__ void resident_quad_drawn(const StepArgs& a, const Ste
         n3 = i3;
         n1 = i1;
     }
-    collide_drawn<SOLID, FORCE>(a, v, q, y, chi, gate, n0, n1, n2, n3, n4, n5, i6, sd, o);
+    collide_drawn<SOLID, FORCE, SAT>(a, v, q, y, chi, gate, n0, n1, n2, n3, n4, n5, i6, sd, o);
     if (RAGGED && m < 4) {
 #pragma unroll
         for (int k = 0; k < 7; ++k) {
@@ -129,13 +129,13 @@ __device__ __forceinline__ void resident_draws(const StepArgs& a, const StepVar&
     gate = FORCE ? rng_block((uint32_t)q, y_key, v.t_lo, v.t_hi, 1u, a.key) : make_uint4(0u, 0u, 0u, 0u);
 }
 
-template <bool SOLID, bool FORCE, bool RAGGED>
+template <bool SOLID, bool FORCE, bool RAGGED, bool SAT = false>
 __device__ __forceinline__ void resident_quad_at(const StepArgs& a, const StepVar& v, const uint32_t* src,
                                                  uint32_t* dst, const uint32_t* Srow, size_t pstride, int lr, int y,
                                                  int q, uint4 (&o)[7]) {
     uint4 chi, gate;
     resident_draws<FORCE>(a, v, q, y, chi, gate);
-    resident_quad_drawn<SOLID, FORCE, RAGGED>(a, v, src, dst, Srow, pstride, lr, y, q, chi, gate, o);
+    resident_quad_drawn<SOLID, FORCE, RAGGED, SAT>(a, v, src, dst, Srow, pstride, lr, y, q, chi, gate, o);
 }
 
 // One step's work items in two classes: the edge items (the rows the

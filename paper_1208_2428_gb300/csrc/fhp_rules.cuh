@@ -10,7 +10,7 @@
 // is replaced by another three-input function of other values of the network
 // that gives the same outputs wherever a difference could be observed, and
 // whatever is no longer used is dropped.  They take 25 (FHP-II), 15 (FHP-I)
-// and 46 (FHP-III) operations, and 30, 18 and 52 with the bounce-back of solid nodes.
+// and 43 (FHP-III) operations, and 30, 18 and 47 with the bounce-back of solid nodes.
 // Every network is equal to its rule table for all node states and both
 // chiralities (compared on the host, tests/test_scatter_logic.py).
 #pragma once
@@ -147,112 +147,104 @@ __host__ __device__ __forceinline__ Planes7 scatter_fhp2_solid(const Planes7& in
     return Planes7{g16, g20, g24, g26, g28, g29, g12};
 }
 
-// FHP-III on fluid nodes: 46 operations.
+// FHP-III on fluid nodes: 43 operations.
 __host__ __device__ __forceinline__ Planes7 scatter_fhp3(const Planes7& in, uint32_t chi) {
-    const uint32_t g0 = lop3<0xC3>(in.m0, in.m3, in.m0);
-    const uint32_t g1 = lop3<0xC3>(in.m2, in.m5, in.m2);
-    const uint32_t g2 = lop3<0xC3>(in.m1, in.m4, in.m1);
-    const uint32_t g3 = lop3<0x81>(g0, g1, g2);
-    const uint32_t g4 = lop3<0x4D>(in.m1, in.m4, in.m5);
-    const uint32_t g5 = lop3<0x1B>(in.m2, in.rest, g3);
-    const uint32_t g6 = lop3<0xA5>(in.m1, g5, g5);
-    const uint32_t g7 = lop3<0x59>(chi, g2, g6);
-    const uint32_t g8 = lop3<0x82>(in.m1, g4, g7);
-    const uint32_t g9 = lop3<0x24>(in.m5, g4, g5);
-    const uint32_t g10 = lop3<0xDB>(in.m1, in.m2, in.m3);
-    const uint32_t g11 = lop3<0xC3>(in.m0, in.m5, in.m0);
-    const uint32_t g12 = lop3<0x24>(in.m0, in.m1, in.m2);
-    const uint32_t g13 = lop3<0x3D>(g10, g11, g12);
-    const uint32_t g14 = lop3<0x93>(chi, g9, g13);
-    const uint32_t g15 = lop3<0x1A>(g2, g9, g14);
-    const uint32_t g16 = lop3<0xDC>(g0, g11, g15);
-    const uint32_t g17 = lop3<0x41>(in.m0, in.m4, g16);
-    const uint32_t g18 = lop3<0xEA>(g7, g12, g17);
-    const uint32_t g19 = lop3<0xA0>(g1, g13, g13);
-    const uint32_t g20 = lop3<0x36>(g0, g18, g19);
-    const uint32_t g21 = lop3<0x2A>(g9, g13, g20);
-    const uint32_t g22 = lop3<0x48>(g1, g8, g21);
-    const uint32_t g23 = lop3<0xB5>(g9, g15, g17);
-    const uint32_t g24 = lop3<0x10>(g6, g10, g18);
-    const uint32_t g25 = lop3<0x14>(in.m3, in.m4, g24);
-    const uint32_t g26 = lop3<0x92>(g1, g23, g25);
-    const uint32_t g27 = lop3<0x27>(g10, g14, g26);
-    const uint32_t g28 = lop3<0x88>(g2, g2, g20);
-    const uint32_t g29 = lop3<0x60>(g25, g27, g28);
-    const uint32_t g30 = lop3<0x5B>(g12, g16, g29);
-    const uint32_t g31 = lop3<0x8E>(g21, g27, g30);
-    const uint32_t g32 = lop3<0x06>(g3, g22, g31);
-    const uint32_t g33 = lop3<0x80>(g0, g19, g20);
-    const uint32_t g34 = lop3<0x7E>(g24, g29, g33);
-    const uint32_t g35 = lop3<0x5A>(in.m3, g34, g34);
-    const uint32_t g36 = lop3<0x69>(g0, g32, g35);
-    const uint32_t g37 = lop3<0xF9>(g22, g23, g29);
-    const uint32_t g38 = lop3<0x3C>(in.m4, g37, in.m4);
-    const uint32_t g39 = lop3<0x69>(g2, g32, g38);
-    const uint32_t g40 = lop3<0x28>(g6, g29, g32);
-    const uint32_t g41 = lop3<0xB6>(g37, g34, g40);
-    const uint32_t g42 = lop3<0xA6>(g2, g29, g41);
-    const uint32_t g43 = lop3<0x96>(in.m2, g32, g42);
-    const uint32_t g44 = lop3<0x5A>(in.m5, g42, g42);
-    const uint32_t g45 = lop3<0x3C>(in.rest, g32, in.rest);
-    return Planes7{g36, g39, g43, g35, g38, g44, g45};
+    const uint32_t g0 = lop3<0xC3>(in.m1, in.m4, in.m1);
+    const uint32_t g1 = lop3<0x82>(in.m0, in.m3, g0);
+    const uint32_t g2 = lop3<0x1B>(in.m2, in.m5, g1);
+    const uint32_t g3 = lop3<0x81>(in.m0, in.m4, g2);
+    const uint32_t g4 = lop3<0x24>(in.m1, in.m2, in.m3);
+    const uint32_t g5 = lop3<0x96>(in.m2, in.m5, g0);
+    const uint32_t g6 = lop3<0x81>(in.m1, in.m3, in.m5);
+    const uint32_t g7 = lop3<0x3A>(g1, g5, g6);
+    const uint32_t g8 = lop3<0xD8>(in.m1, in.m3, chi);
+    const uint32_t g9 = lop3<0x48>(in.rest, g7, g8);
+    const uint32_t g10 = lop3<0xBE>(g3, g4, g9);
+    const uint32_t g11 = lop3<0x82>(in.m4, in.rest, g10);
+    const uint32_t g12 = lop3<0x81>(in.m0, in.m2, in.m4);
+    const uint32_t g13 = lop3<0x96>(g6, g10, g12);
+    const uint32_t g14 = lop3<0x82>(in.rest, g2, g13);
+    const uint32_t g15 = lop3<0x69>(in.m1, chi, g11);
+    const uint32_t g16 = lop3<0x69>(in.m5, g6, g15);
+    const uint32_t g17 = lop3<0x09>(g1, g6, g12);
+    const uint32_t g18 = lop3<0xA4>(g13, g16, g17);
+    const uint32_t g19 = lop3<0x82>(g2, g8, g18);
+    const uint32_t g20 = lop3<0x70>(g4, g9, g18);
+    const uint32_t g21 = lop3<0x9E>(g14, g19, g20);
+    const uint32_t g22 = lop3<0x78>(g10, g12, g14);
+    const uint32_t g23 = lop3<0x70>(g22, g16, g17);
+    const uint32_t g24 = lop3<0xC6>(g11, g21, g23);
+    const uint32_t g25 = lop3<0x5A>(g0, g23, g23);
+    const uint32_t g26 = lop3<0x96>(g2, g8, g16);
+    const uint32_t g27 = lop3<0xC9>(g24, g25, g26);
+    const uint32_t g28 = lop3<0x98>(g11, g21, g27);
+    const uint32_t g29 = lop3<0x92>(g1, g13, g24);
+    const uint32_t g30 = lop3<0xBA>(g4, g25, g29);
+    const uint32_t g31 = lop3<0xE4>(in.m2, in.m4, g19);
+    const uint32_t g32 = lop3<0x5A>(in.m0, g31, g31);
+    const uint32_t g33 = lop3<0x86>(g17, g30, g32);
+    const uint32_t g34 = lop3<0xD4>(g28, g30, g33);
+    const uint32_t g35 = lop3<0x78>(g24, g25, g34);
+    const uint32_t g36 = lop3<0x5A>(in.m0, g35, g35);
+    const uint32_t g37 = lop3<0x5A>(in.m1, g34, g34);
+    const uint32_t g38 = lop3<0x5A>(in.m2, g21, g21);
+    const uint32_t g39 = lop3<0x96>(in.m3, g23, g35);
+    const uint32_t g40 = lop3<0x99>(g25, g25, g37);
+    const uint32_t g41 = lop3<0x96>(g5, g25, g38);
+    const uint32_t g42 = lop3<0x5A>(in.rest, g23, g23);
+    return Planes7{g36, g37, g38, g39, g40, g41, g42};
 }
 
-// FHP-III, bounce-back on solid nodes: 52 operations.
+// FHP-III, bounce-back on solid nodes: 47 operations.
 __host__ __device__ __forceinline__ Planes7 scatter_fhp3_solid(const Planes7& in, uint32_t chi, uint32_t solid) {
-    const uint32_t g0 = lop3<0xC3>(in.m0, in.m3, in.m0);
-    const uint32_t g1 = lop3<0xC3>(in.m2, in.m5, in.m2);
-    const uint32_t g2 = lop3<0xC3>(in.m1, in.m4, in.m1);
-    const uint32_t g3 = lop3<0x81>(g0, g1, g2);
-    const uint32_t g4 = lop3<0x1B>(in.m2, in.rest, g3);
-    const uint32_t g5 = lop3<0xA5>(in.m1, g4, g4);
-    const uint32_t g6 = lop3<0x59>(chi, g2, g5);
-    const uint32_t g7 = lop3<0x27>(in.m1, in.m5, g2);
-    const uint32_t g8 = lop3<0x42>(in.m5, g4, g7);
-    const uint32_t g9 = lop3<0x48>(g5, g6, g8);
-    const uint32_t g10 = lop3<0xDB>(in.m1, in.m2, in.m3);
-    const uint32_t g11 = lop3<0xC3>(in.m0, in.m5, in.m0);
-    const uint32_t g12 = lop3<0x77>(g10, g10, g11);
-    const uint32_t g13 = lop3<0x24>(in.m0, in.m1, in.m2);
-    const uint32_t g14 = lop3<0x93>(chi, g8, g12);
-    const uint32_t g15 = lop3<0x1A>(g2, g8, g14);
-    const uint32_t g16 = lop3<0xDC>(g0, g11, g15);
-    const uint32_t g17 = lop3<0x41>(in.m0, in.m4, g16);
-    const uint32_t g18 = lop3<0xEA>(g6, g13, g17);
-    const uint32_t g19 = lop3<0x88>(g1, g1, g12);
-    const uint32_t g20 = lop3<0x36>(g0, g18, g19);
-    const uint32_t g21 = lop3<0x2A>(g8, g12, g20);
-    const uint32_t g22 = lop3<0x48>(g1, g9, g21);
-    const uint32_t g23 = lop3<0xB5>(g8, g15, g17);
-    const uint32_t g24 = lop3<0x10>(g5, g10, g18);
-    const uint32_t g25 = lop3<0x14>(in.m3, in.m4, g24);
-    const uint32_t g26 = lop3<0x82>(g1, g23, g25);
-    const uint32_t g27 = lop3<0x27>(g10, g14, g26);
-    const uint32_t g28 = lop3<0xA0>(g2, g20, g20);
-    const uint32_t g29 = lop3<0x60>(g25, g27, g28);
-    const uint32_t g30 = lop3<0x5B>(g13, g16, g29);
-    const uint32_t g31 = lop3<0x8E>(g21, g27, g30);
-    const uint32_t g32 = lop3<0x46>(g3, g22, g31);
-    const uint32_t g33 = lop3<0x20>(g0, g18, g19);
-    const uint32_t g34 = lop3<0x3E>(g24, g29, g33);
-    const uint32_t g35 = lop3<0x96>(in.m0, g32, g34);
-    const uint32_t g36 = lop3<0xE2>(in.m3, solid, g35);
-    const uint32_t g37 = lop3<0xFB>(g22, g23, g29);
-    const uint32_t g38 = lop3<0x96>(in.m1, g32, g37);
-    const uint32_t g39 = lop3<0xE2>(in.m4, solid, g38);
-    const uint32_t g40 = lop3<0x28>(g5, g29, g32);
-    const uint32_t g41 = lop3<0x9E>(g34, g37, g40);
-    const uint32_t g42 = lop3<0xA6>(g2, g29, g41);
-    const uint32_t g43 = lop3<0x96>(in.m2, g32, g42);
-    const uint32_t g44 = lop3<0xE2>(in.m5, solid, g43);
-    const uint32_t g45 = lop3<0x5A>(in.m3, g34, g34);
-    const uint32_t g46 = lop3<0xE2>(in.m0, solid, g45);
-    const uint32_t g47 = lop3<0x5A>(in.m4, g37, g37);
-    const uint32_t g48 = lop3<0xE2>(in.m1, solid, g47);
-    const uint32_t g49 = lop3<0x3C>(in.m5, g42, in.m5);
-    const uint32_t g50 = lop3<0xE2>(in.m2, solid, g49);
-    const uint32_t g51 = lop3<0xD2>(in.rest, solid, g32);
-    return Planes7{g36, g39, g44, g46, g48, g50, g51};
+    const uint32_t g0 = lop3<0x24>(in.m1, in.m2, in.m3);
+    const uint32_t g1 = lop3<0xC3>(in.m1, in.m4, in.m1);
+    const uint32_t g2 = lop3<0x82>(in.m0, in.m3, g1);
+    const uint32_t g3 = lop3<0x1B>(in.m2, in.m5, g2);
+    const uint32_t g4 = lop3<0x81>(in.m0, in.m4, g3);
+    const uint32_t g5 = lop3<0x96>(in.m2, in.m5, g1);
+    const uint32_t g6 = lop3<0x81>(in.m1, in.m3, in.m5);
+    const uint32_t g7 = lop3<0x3A>(g2, g5, g6);
+    const uint32_t g8 = lop3<0xD8>(in.m1, in.m3, chi);
+    const uint32_t g9 = lop3<0x48>(in.rest, g7, g8);
+    const uint32_t g10 = lop3<0xBE>(g0, g4, g9);
+    const uint32_t g11 = lop3<0x82>(in.m4, in.rest, g10);
+    const uint32_t g12 = lop3<0x81>(in.m0, in.m2, in.m4);
+    const uint32_t g13 = lop3<0x96>(g6, g10, g12);
+    const uint32_t g14 = lop3<0x82>(in.rest, g3, g13);
+    const uint32_t g15 = lop3<0x69>(in.m1, chi, g11);
+    const uint32_t g16 = lop3<0x96>(g3, g7, g15);
+    const uint32_t g17 = lop3<0x09>(g2, g6, g12);
+    const uint32_t g18 = lop3<0xA4>(g13, g16, g17);
+    const uint32_t g19 = lop3<0x82>(g3, g8, g18);
+    const uint32_t g20 = lop3<0x70>(g0, g9, g18);
+    const uint32_t g21 = lop3<0x9E>(g14, g19, g20);
+    const uint32_t g22 = lop3<0x78>(g10, g12, g14);
+    const uint32_t g23 = lop3<0x2A>(g16, g17, g22);
+    const uint32_t g24 = lop3<0xC6>(g11, g21, g23);
+    const uint32_t g25 = lop3<0xC6>(solid, g1, g23);
+    const uint32_t g26 = lop3<0x96>(g7, g8, g15);
+    const uint32_t g27 = lop3<0xC9>(g24, g25, g26);
+    const uint32_t g28 = lop3<0x98>(g11, g21, g27);
+    const uint32_t g29 = lop3<0x98>(g2, g9, g24);
+    const uint32_t g30 = lop3<0xBA>(g0, g25, g29);
+    const uint32_t g31 = lop3<0x3C>(in.m2, g21, in.m2);
+    const uint32_t g32 = lop3<0x74>(in.m4, g19, g31);
+    const uint32_t g33 = lop3<0x3C>(in.m0, g32, in.m0);
+    const uint32_t g34 = lop3<0x29>(g17, g28, g33);
+    const uint32_t g35 = lop3<0xD4>(g28, g30, g34);
+    const uint32_t g36 = lop3<0x78>(g24, g25, g35);
+    const uint32_t g37 = lop3<0x5A>(in.m0, g36, g36);
+    const uint32_t g38 = lop3<0xE2>(in.m3, solid, g37);
+    const uint32_t g39 = lop3<0x3C>(in.m1, g35, in.m1);
+    const uint32_t g40 = lop3<0xE2>(in.m4, solid, g39);
+    const uint32_t g41 = lop3<0xE2>(in.m5, solid, g31);
+    const uint32_t g42 = lop3<0x96>(in.m3, g23, g36);
+    const uint32_t g43 = lop3<0xE2>(in.m0, solid, g42);
+    const uint32_t g44 = lop3<0xC3>(g25, g40, g25);
+    const uint32_t g45 = lop3<0x96>(g5, g25, g41);
+    const uint32_t g46 = lop3<0x96>(in.rest, g1, g25);
+    return Planes7{g38, g40, g41, g43, g44, g45, g46};
 }
 
 }  // namespace fhp
