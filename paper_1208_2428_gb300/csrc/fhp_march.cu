@@ -83,12 +83,11 @@ bool march_supported(const Geometry& g, int k) {
 
 // Where register marching is the automatic choice (GB300, GSUPS, marching
 // against the kernel it replaces; the lattices hold a cylinder):
-//   without forcing   12288 x 1024: 2.9 against 2.5 thousand; 4096 x 4096 4.1
-//     against 3.2; 8192 x 4096 4.8 (k = 2; 4.2 with k = 3) against 3.8;
-//     16384 x 4096 6.6 (k = 3; 6.0 with k = 2) against 4.0; 29,984 x 27,990
-//     7.8 against 3.3; but 4096 x 2048 2.9 against 3.1 (resident in shared
-//     memory): from 12 million nodes on, and k = 2 between 24 and 48 million,
-//     where the rows of a band are too few for a third level;
+//   without forcing   8192 x 2560: 3.8 thousand with k = 2 (3.7 with k = 3)
+//     against 3.3; 8192 x 4096 4.8 (4.4) against 3.8; 16384 x 4096 6.1 with k = 3
+//     (5.3 with k = 2) against 4.0; 29,984 x 27,990 7.6 (5.5) against 3.3: from 12
+//     million nodes on (smaller ones are resident in shared memory anyway),
+//     k = 3 from 48 million, where the bands are high enough for a third level;
 //   with forcing (p = 5e-4)   12288 x 4096 3.8 against 3.4, 16384 x 4096 4.1
 //     against 3.6, 29,984 x 27,990 4.8 against 3.0, but 8192 x 4096 3.5 against
 //     3.7: from 40 million nodes, k = 2 (k = 3 has 12 warps an SM to hide the
@@ -104,7 +103,7 @@ int march_choice(const Geometry& g, const ForcingTable& ft, bool force) {
         return rare && nodes >= (g.rules == 3 ? 200000000LL : 40000000LL) ? 2 : 0;
     }
     if (nodes < 12000000) return 0;
-    return nodes >= 24000000 && nodes < 48000000 ? 2 : 3;
+    return nodes < 48000000 ? 2 : 3;
 }
 
 cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const uint32_t* solid, bool has_solid,

@@ -66,7 +66,7 @@ def test_march_every_candidate_forced_and_full(pkg, oracle_mod):
         assert np.array_equal(got, want)
 
 
-@pytest.mark.parametrize("W,H,p,block", [(8192, 2560, 0.0, 3), (8192, 4096, 0.0, 2), (16384, 2560, 5e-4, 2),
+@pytest.mark.parametrize("W,H,p,block", [(8192, 2560, 0.0, 2), (16384, 4096, 0.0, 3), (16384, 2560, 5e-4, 2),
                                          (12032, 3400, 1e-3, 2)])
 def test_automatic_choice_equals_direct_kernel(pkg, W, H, p, block):
     import torch
