@@ -169,7 +169,8 @@ FHP_API int fhp_set_forcing(fhp_lattice* lattice, double p);
  * lattices) use the single-step kernels.  With step kernel 4 (resident) the
  * value is instead the number of steps between exchanges of strip rows: 2
  * selects the two-ghost-row variant where every strip holds at least 4 rows,
- * other values the one-row exchange.  Results are identical for every value.
+ * other values the one-row exchange (the automatic choice of kernel 4 also
+ * chooses among 1, 2 and 4 steps between exchanges).  Results are identical for every value.
  * Default 1. */
 FHP_API int fhp_set_temporal_block(fhp_lattice* lattice, int32_t k);
 
@@ -236,7 +237,7 @@ FHP_API int fhp_get_rows_device(fhp_lattice* lattice, int32_t y0, int32_t n, uin
 FHP_API int fhp_set_rows_device(fhp_lattice* lattice, int32_t y0, int32_t n, const uint32_t* device_words);
 
 /* Temporal block fhp_step will use (1 if blocking is off or unsupported for
- * this lattice; for the resident kernel the exchange interval, 1 or 2), or
+ * this lattice; for the resident kernel the exchange interval, 1, 2 or 4), or
  * -1 for a NULL lattice. */
 FHP_API int fhp_get_temporal_block(const fhp_lattice* lattice);
 
@@ -253,7 +254,7 @@ FHP_API int fhp_get_temporal_block_kernel(const fhp_lattice* lattice);
 
 /* Autotuner.  Times every step configuration that applies to this lattice --
  * direct, ring, multi-step and resident kernels (the resident one with
- * exchanges every step and every second step), and temporal blocks
+ * exchanges every step, second and fourth step), and temporal blocks
  * k = 2, 3, 4, 8 --
  * over trial_steps steps each (a multiple of 8 in [8, 4096]; each candidate
  * runs once untimed, then timed with CUDA events on the lattice's stream) and

@@ -65,8 +65,9 @@ struct TuneKey {
 struct TuneChoice {
     int kernel;   // fhp::StepKernel other than kStepAuto
     int k;        // temporal block
-    int bk;       // temporal-block kernel (0 automatic, 1 row wavefronts, 2 tiles, 3 register marching)
+    int bk;       // temporal-block kernel (0 automatic, 1 row wavefronts, 2 tiles, 3 register marching), or kAutoInterval
 };
+constexpr int kAutoInterval = 4;   // TuneChoice::bk: resident kernel, k steps between exchanges
 std::mutex g_tune_mutex;
 std::vector<std::pair<TuneKey, TuneChoice>> g_tuned;
 
@@ -164,9 +165,9 @@ struct DeviceGuard {
 // while they are automatic (kernel 0, k = 1), the configuration autotuned
 // for this shape if there is one, else the shared-memory resident kernel for
 // every lattice it holds (us a step, p = 1e-3, against the multi-step ring: 512 x
-// 512 1.6 against 4.4, 4096 x 1024 1.9 against 4.2, 4096 x 3072 3.3 against 5.5,
-// 4096 x 4096 3.7 against register marching's 5.7), else register marching for the lattices it
-// is fastest on (fhp::march_choice), else the kernel of
+// 512 1.5 against 4.4, 4096 x 1024 1.9 against 4.2, 4096 x 3072 3.3 against 5.5,
+// 4096 x 4096 3.7 against register marching's 5.7), else register marching for
+// the lattices it is fastest on (fhp::march_choice), else the kernel of
 // fhp::resolved_step_kernel.
 void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk = nullptr) {
     *kernel = h->step_kernel;
@@ -180,8 +181,10 @@ void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk
         if (bk) *bk = c.bk;
         return;
     }
-    if (fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 1)) {
+    if (const int gh = fhp::resident_interval_for(h->g, h->has_solid, h->staging_bytes, h->force)) {
         *kernel = fhp::kStepResident;
+        *k_block = gh;
+        if (bk) *bk = kAutoInterval;
         return;
     }
     if (const int mk = fhp::march_choice(h->g, h->ft, h->force)) {
@@ -196,11 +199,19 @@ int reported_kernel(const fhp_lattice* h, int kernel) {
     return h->g.rules == 3 && kernel == fhp::kStepResident ? fhp::kStepRun : kernel;
 }
 
-// Steps between exchanges of the resident kernel for these settings (2 when
-// asked for and supported, else 1), or 0 if the resident kernel does not run.
-int resident_interval(const fhp_lattice* h, int kernel, int k_block) {
+// Steps between exchanges of the resident kernel for these settings, or 0 if
+// the resident kernel does not run: k_block as it is where the library chose it
+// (bk = kAutoInterval); else 2 when asked for and one strip per SM would hold
+// at least 4 rows, else 1.
+int resident_interval(const fhp_lattice* h, int kernel, int k_block, int bk) {
     if (kernel != fhp::kStepResident) return 0;
-    if (k_block == 2 && fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 2)) return 2;
+    if (bk == kAutoInterval) return k_block;
+    int sms = 0;
+    if (k_block == 2 && h->g.rules != 3 &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess &&
+        h->g.H / (h->g.H < sms ? h->g.H : sms) >= 4 &&
+        fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 2))
+        return 2;
     return fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 1) ? 1 : 0;
 }
 
@@ -520,7 +531,7 @@ int fhp_step(fhp_lattice* h, int64_t n) {
     const fhp::Key2 key{(uint32_t)h->seed, (uint32_t)(h->seed >> 32)};
     int kernel = h->step_kernel, k_block = h->k_block, bk = h->block_kernel;
     effective_settings(h, &kernel, &k_block, &bk);
-    int gh = resident_interval(h, kernel, k_block);
+    int gh = resident_interval(h, kernel, k_block, bk);
     if (gh > 0 && n <= 3 && h->step_kernel == fhp::kStepAuto) {
         // Up to three steps do not repay moving the lattice into shared memory
         // and back (about 10 us; a direct step of such a lattice takes 4 to 6).
@@ -530,14 +541,13 @@ int fhp_step(fhp_lattice* h, int64_t n) {
     }
     if (gh > 0) {
         // The lattice stays in shared memory for launches of up to 2^24 steps
-        // (exchange rows in the byte-staging area, step counters in the tile
-        // counters).
+        // (exchange rows in the byte-staging area).
         int64_t left = n;
         while (left > 0) {
             const int chunk = (int)(left < (1 << 24) ? left : (1 << 24));
             cudaError_t e = fhp::launch_resident(h->g, h->buf[h->cur], h->buf[h->cur ^ 1], h->solid, h->has_solid,
                                                  h->force, h->ft, key, (uint64_t)h->t, chunk, gh,
-                                                 reinterpret_cast<uint32_t*>(h->staging), h->tile_done, h->stream,
+                                                 reinterpret_cast<uint32_t*>(h->staging), h->staging_bytes, h->stream,
                                                  h->flags + 1);
             if (e != cudaSuccess) return cuda_fail(h, e, "launching the resident kernel");
             ++h->launches;
@@ -736,7 +746,7 @@ int fhp_get_temporal_block(const fhp_lattice* h) {
     if (!h) return -1;
     int kernel, k_block, bk;
     effective_settings(h, &kernel, &k_block, &bk);
-    const int gh = resident_interval(h, kernel, k_block);
+    const int gh = resident_interval(h, kernel, k_block, bk);
     if (gh > 0) return gh;
     return blocked_kind(h, k_block, bk) != 0 ? k_block : 1;
 }
@@ -752,7 +762,7 @@ int fhp_get_temporal_block_kernel(const fhp_lattice* h) {
     if (!h) return -1;
     int kernel, k_block, bk;
     effective_settings(h, &kernel, &k_block, &bk);
-    if (resident_interval(h, kernel, k_block) > 0) return 0;
+    if (resident_interval(h, kernel, k_block, bk) > 0) return 0;
     return blocked_kind(h, k_block, bk);
 }
 
@@ -785,10 +795,9 @@ int fhp_autotune(fhp_lattice* h, int32_t trial_steps, int32_t* out_kernel, int32
         cands.push_back({fhp::kStepRing, 1, 0});
         cands.push_back({fhp::kStepRun, 1, 0});
     }
-    if (fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 1))
-        cands.push_back({fhp::kStepResident, 1, 0});
-    if (fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, 2))
-        cands.push_back({fhp::kStepResident, 2, 0});
+    for (int gh : {1, 2, 4})
+        if ((gh == 1 || h->g.rules != 3) && fhp::resident_supported(h->g, h->has_solid, h->staging_bytes, gh))
+            cands.push_back({fhp::kStepResident, gh, kAutoInterval});
     // Temporal blocks (trial_steps mod k steps run one at a time): row
     // wavefronts and 2-D tiles, where each supports the lattice.
     for (int k : {2, 3, 4})
