@@ -1420,18 +1420,33 @@ bool marches(const Member& m, int k) {
     return m.used && fhp::march_supported(m.g, k) && m.ft.p_plus_1 <= (1ull << 32) / 100;
 }
 
-// Steps per pass: 3 without forcing, except for batches whose bands would be
-// too low for a third level (see fhp::march_choice); 0 if no member marches.
-int march_block(const fhp_batch* b) {
-    long long nodes = 0;
-    bool force = false;
-    for (const Member& m : b->members) {
-        if (!marches(m, 2)) continue;
-        nodes += (long long)m.g.W * m.g.H;
-        force = force || m.ft.q[32] != 0;
-    }
-    if (nodes == 0) return 0;
+// Steps per pass for marching members of that many nodes together: 3 without
+// forcing, except where the bands would be too low for a third level (24 to 48
+// million nodes: 8192 x 4096 4.8 thousand GSUPS with k = 2, 4.4 with k = 3).
+int march_block_for(long long nodes, bool force) {
     return force || (nodes >= 24000000 && nodes < 48000000) ? 2 : 3;
+}
+
+// Nodes of the marching members without and with forcing.
+void march_nodes(const fhp_batch* b, long long& plain, long long& forced) {
+    plain = forced = 0;
+    for (const Member& m : b->members)
+        if (marches(m, 2)) (m.ft.q[32] != 0 ? forced : plain) += (long long)m.g.W * m.g.H;
+}
+
+// Members with and without forcing march in launches of their own where each
+// kind fills the machine by itself: the walks of the one and the passes of 3
+// steps of the other then set their own pace (24 lattices of 256 .. 8192 nodes a
+// side, half of them forced: 3990 GSUPS against 3360 in one launch).
+bool march_split(long long plain, long long forced) { return plain >= 16000000 && forced >= 16000000; }
+
+// The largest number of steps per pass a call of the batch would use (0: no
+// member marches).
+int march_block(const fhp_batch* b) {
+    long long plain, forced;
+    march_nodes(b, plain, forced);
+    if (plain + forced == 0) return 0;
+    return march_split(plain, forced) ? march_block_for(plain, false) : march_block_for(plain + forced, forced > 0);
 }
 
 // One cooperative launch per group of members: member i advances by
@@ -1539,10 +1554,10 @@ int launch_march_passes(fhp_batch* b, int k, const std::vector<int>& passes) {
 }
 
 // One chunk by register marching: the members that march advance by passes of
-// k steps (k = 3: the remainder by up to two passes of 2), the steps left over
+// 2 or 3 steps (3: the remainder by up to two passes of 2), the steps left over
 // (all steps of the other members) run on the batch step kernel `kind`.  The
 // result equals single steps for every member.
-int run_march_chunk(fhp_batch* b, int chunk, int k, int kind, std::vector<int>& steps_of, double* updates) {
+int run_march_chunk(fhp_batch* b, int chunk, int kind, std::vector<int>& steps_of, double* updates) {
     const size_t nm = b->members.size();
     if (!reserve_march(b)) return run_chunk(b, chunk, kind, steps_of, updates);
     std::vector<int> left(nm, 0), passes(nm, 0);
@@ -1556,21 +1571,36 @@ int run_march_chunk(fhp_batch* b, int chunk, int k, int kind, std::vector<int>& 
         left[i] = steps_of[i] = (int)s;
         upd += (double)m.g.W * m.g.H * (double)s;
     }
-    for (; k >= 2; --k) {
-        bool any = false;
-        for (size_t i = 0; i < nm; ++i) {
-            passes[i] = 0;
-            if (left[i] < 2 || !marches(b->members[i], k)) continue;
-            // k = 3: what remains is even (1 step is 2 + 2 less a pass of 3).
-            passes[i] = k == 2 ? left[i] / 2 : left[i] % 3 == 1 ? (left[i] - 4) / 3 : left[i] / 3;
-            if (passes[i] < 0) passes[i] = 0;
-            left[i] -= passes[i] * k;
-            any = any || passes[i] > 0;
+    // The members of one kind (-1: all), passes of k steps downwards.
+    auto run = [&](int forced, int k) -> int {
+        for (; k >= 2; --k) {
+            bool any = false;
+            for (size_t i = 0; i < nm; ++i) {
+                const Member& m = b->members[i];
+                passes[i] = 0;
+                if (left[i] < 2 || !marches(m, k) || (forced >= 0 && (m.ft.q[32] != 0) != (forced != 0))) continue;
+                // k = 3: what remains is even (1 step is 2 + 2 less a pass of 3).
+                passes[i] = k == 2 ? left[i] / 2 : left[i] % 3 == 1 ? (left[i] - 4) / 3 : left[i] / 3;
+                if (passes[i] < 0) passes[i] = 0;
+                left[i] -= passes[i] * k;
+                any = any || passes[i] > 0;
+            }
+            if (!any) continue;
+            const int rc = launch_march_passes(b, k, passes);
+            if (rc != FHP_OK) return rc;
         }
-        if (!any) continue;
-        const int rc = launch_march_passes(b, k, passes);
-        if (rc != FHP_OK) return rc;
+        return FHP_OK;
+    };
+    long long plain, forced;
+    march_nodes(b, plain, forced);
+    int mrc;
+    if (march_split(plain, forced)) {
+        mrc = run(0, march_block_for(plain, false));
+        if (mrc == FHP_OK) mrc = run(1, 2);
+    } else {
+        mrc = run(-1, march_block_for(plain + forced, forced > 0));
     }
+    if (mrc != FHP_OK) return mrc;
     std::vector<int> rest_of;
     const int rc = run_chunk(b, chunk, kind, rest_of, nullptr, &left);
     if (rc != FHP_OK) return rc;
@@ -1682,7 +1712,7 @@ int batch_step(fhp_batch* b, int64_t n) {
                 if (rc != FHP_OK) return rc;
                 cudaEventRecord(tr.ev[k][0], b->stream);
                 tr.updates[k] = 0.0;
-                rc = tr.march[k]   ? run_march_chunk(b, part, tr.block[k], tr.kind[k], steps_of, &tr.updates[k])
+                rc = tr.march[k]   ? run_march_chunk(b, part, tr.kind[k], steps_of, &tr.updates[k])
                      : tr.block[k] > 1 ? run_blocked_chunk(b, part, tr.block[k], tr.kind[k], steps_of, &tr.updates[k])
                                        : run_chunk(b, part, tr.kind[k], steps_of, &tr.updates[k]);
                 if (rc != FHP_OK) return rc;
@@ -1723,11 +1753,11 @@ int batch_step(fhp_batch* b, int64_t n) {
             } else {
                 march = chunk >= 2 && reserve_march(b);
             }
-            if (march) k = march_block(b);   // (the members may have changed since the trial)
-            march = march && k != 0;
+            march = march && march_block(b) != 0;   // (the members may have changed since the trial)
+            if (!march && b->tuned_march[cls]) k = 1;
         }
         if (k == 0) k = 1;
-        rc = march   ? run_march_chunk(b, chunk, k, kind, steps_of, nullptr)
+        rc = march   ? run_march_chunk(b, chunk, kind, steps_of, nullptr)
              : k > 1 ? run_blocked_chunk(b, chunk, k, kind, steps_of, nullptr)
                      : run_chunk(b, chunk, kind, steps_of, nullptr);
         if (rc != FHP_OK) return rc;
