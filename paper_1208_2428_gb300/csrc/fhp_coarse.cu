@@ -9,11 +9,16 @@
 // with the integer momenta jx2 = sum_i n_i 2cos(theta_i) and
 // jy = sum_i n_i sgn(sin(theta_i)), theta_i = (i-2)*60 degrees.
 //
-// The planes are read once, at the speed of memory: a CTA takes the row of
-// blocks that 32 neighbouring words hold (one block where a block is wider),
-// its eight warps take the blocks' rows in turn, and a lane counts down its
-// word column, so every load is one row segment of a plane.  16384 x 4096,
-// B = 64: 23.6 us; 49 us when one warp gathered the words of one block.
+// The planes are read once: a CTA takes the row of blocks that a stretch of a
+// row holds, its warps take the blocks' rows in turn, and a lane counts down its
+// column, so every load is one row segment of a plane.  Where blocks and quads
+// of four words fit each other (1, 2 or a multiple of 4 words per block) a
+// lane's column is a quad and a load of a warp 512 bytes; else it is a word.
+// The latency of the loads bounds it, so 16 warps take two rows at a time:
+// 16384 x 4096, B = 64 (call and flushed caches): 15.3 us; 23.5 us with 8 warps
+// and one row at a time
+// (and with words); 49 us when one warp gathered the words of one block.
+// Repeated, in L2: B = 32 12.5 us, 64 8.4, 128 10.3, 256 14.4.
 #include "fhp_internal.h"
 
 namespace fhp {
@@ -21,6 +26,35 @@ namespace {
 
 constexpr int kBlock = 256;
 constexpr int kWarps = kBlock / 32;
+constexpr int kQuadBlock = 512;
+constexpr int kQuadWarps = kQuadBlock / 32;
+
+// Counts and derived fields of one block from its seven particle counts and its
+// fluid nodes.
+__device__ __forceinline__ void write_cell(long long cell, const unsigned (&n)[8], int32_t* __restrict__ counts,
+                                           float* __restrict__ rho, float* __restrict__ ux, float* __restrict__ uy) {
+    long long mass = 0;
+    for (int k = 0; k < 7; ++k) mass += n[k];
+    const long long jx2 = -(long long)n[0] + n[1] + 2LL * n[2] + n[3] - (long long)n[4] - 2LL * n[5];
+    const long long jy = -(long long)n[0] - (long long)n[1] + n[3] + n[4];
+    int32_t* c = counts + (size_t)cell * 9;
+    for (int k = 0; k < 7; ++k) c[k] = (int32_t)n[k];
+    c[7] = (int32_t)n[7];
+    c[8] = (int32_t)mass;
+    const double half_sqrt3 = sqrt(3.0) * 0.5;
+    const double vy = mass ? half_sqrt3 * (double)jy / (double)mass : 0.0;
+    uy[cell] = __double2float_rn(vy);
+    if (mass < (1 << 23) && n[7] <= (1u << 24)) {
+        // Quotients of integers that a float holds exactly: the float division
+        // gives what the double one rounded to float gives (53 >= 2 * 24 + 2
+        // bits), without two of the three divisions on the few double units.
+        rho[cell] = n[7] ? __fdiv_rn((float)mass, (float)n[7]) : 0.0f;
+        ux[cell] = mass ? __fdiv_rn((float)jx2, (float)(2 * mass)) : 0.0f;
+        return;
+    }
+    rho[cell] = __double2float_rn(n[7] ? (double)mass / (double)n[7] : 0.0);
+    ux[cell] = __double2float_rn((double)jx2 / (2.0 * (double)mass));
+}
 
 // Bw words per block row, nb blocks per CTA (nb * Bw <= 32, or nb = 1).
 template <bool SOLID>
@@ -60,7 +94,6 @@ __global__ void __launch_bounds__(kBlock) coarse_kernel(Geometry g, const uint32
     __syncthreads();
     const int j = (int)threadIdx.x;
     if (j >= nb || bx0 + j >= nbx) return;
-    unsigned fluid = 0;
     const int width = min(Bw, 32);
 #pragma unroll
     for (int k = 0; k < 8; ++k) n[k] = 0;
@@ -68,23 +101,90 @@ __global__ void __launch_bounds__(kBlock) coarse_kernel(Geometry g, const uint32
 #pragma unroll
         for (int k = 0; k < 8; ++k) n[k] += part[0][k][j * Bw + c];
     }
-    fluid = n[7];
     const long long cell = (long long)by * nbx + bx0 + j;
-    long long mass = 0;
-    for (int k = 0; k < 7; ++k) mass += n[k];
-    const long long jx2 = -(long long)n[0] + n[1] + 2LL * n[2] + n[3] - (long long)n[4] - 2LL * n[5];
-    const long long jy = -(long long)n[0] - (long long)n[1] + n[3] + n[4];
-    int32_t* c = counts + (size_t)cell * 9;
-    for (int k = 0; k < 7; ++k) c[k] = (int32_t)n[k];
-    c[7] = (int32_t)fluid;
-    c[8] = (int32_t)mass;
-    const double half_sqrt3 = sqrt(3.0) * 0.5;
-    const double r = fluid ? (double)mass / (double)fluid : 0.0;
-    const double vx = mass ? (double)jx2 / (2.0 * (double)mass) : 0.0;
-    const double vy = mass ? half_sqrt3 * (double)jy / (double)mass : 0.0;
-    rho[cell] = __double2float_rn(r);
-    ux[cell] = __double2float_rn(vx);
-    uy[cell] = __double2float_rn(vy);
+    write_cell(cell, n, counts, rho, ux, uy);
+}
+
+// Quads: a lane counts PER blocks of its four words (4, 2 or 1); `lanes` lanes
+// hold one block where PER is 1.
+template <bool SOLID, int PER>
+__global__ void __launch_bounds__(kQuadBlock, 2) coarse_quads_kernel(Geometry g, const uint32_t* __restrict__ state,
+                                                              const uint32_t* __restrict__ solid, int B, int lanes,
+                                                              int groups, int32_t* __restrict__ counts,
+                                                              float* __restrict__ rho, float* __restrict__ ux,
+                                                              float* __restrict__ uy) {
+    __shared__ unsigned part[8 * PER][32 + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nbx = g.W / B;
+    const int by = (int)(blockIdx.x / (unsigned)groups), group = (int)(blockIdx.x - (unsigned)by * (unsigned)groups);
+    const int width = PER == 1 ? lanes * max(1, 32 / lanes) : 32;   // quads of the CTA
+    const int q0 = group * width, quads = min(width, g.nq - q0);
+    unsigned n[PER][8];
+#pragma unroll
+    for (int b = 0; b < PER; ++b)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) n[b][k] = 0u;
+    auto add = [&](const uint4& v, int k) {
+        if (PER == 4) {
+            n[0][k] += __popc(v.x);
+            n[1 % PER][k] += __popc(v.y);
+            n[2 % PER][k] += __popc(v.z);
+            n[3 % PER][k] += __popc(v.w);
+        } else if (PER == 2) {
+            n[0][k] += __popc(v.x) + __popc(v.y);
+            n[1 % PER][k] += __popc(v.z) + __popc(v.w);
+        } else {
+            n[0][k] += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        }
+    };
+    for (int c = lane; c < quads; c += 32) {
+        const size_t base = (size_t)by * B * g.Pq + 4 * (size_t)(q0 + c);
+        // (B is a multiple of 32 and a warp takes every 16th row: pairs of rows
+        // where the counters leave the registers for it.)
+        constexpr int ROWS = PER == 4 ? 1 : 2;
+        for (int r = warp; r < B; r += ROWS * kQuadWarps) {
+            uint4 p[ROWS][7], f[ROWS];
+#pragma unroll
+            for (int h = 0; h < ROWS; ++h) {
+                const size_t off = base + (size_t)(r + h * kQuadWarps) * g.Pq;
+                f[h] = SOLID ? *reinterpret_cast<const uint4*>(solid + off) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int k = 0; k < 7; ++k)
+                    p[h][k] = *reinterpret_cast<const uint4*>(state + (size_t)k * g.plane_words + off);
+            }
+#pragma unroll
+            for (int h = 0; h < ROWS; ++h) {
+                add(make_uint4(~f[h].x, ~f[h].y, ~f[h].z, ~f[h].w), 7);
+#pragma unroll
+                for (int k = 0; k < 7; ++k)
+                    add(make_uint4(p[h][k].x & ~f[h].x, p[h][k].y & ~f[h].y, p[h][k].z & ~f[h].z,
+                                   p[h][k].w & ~f[h].w), k);
+            }
+        }
+    }
+    for (int i = threadIdx.x; i < 8 * PER * 33; i += kQuadBlock) part[i / 33][i % 33] = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < PER; ++b)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) atomicAdd(&part[8 * b + k][lane], n[b][k]);
+    __syncthreads();
+    // Thread j writes block j of the CTA.
+    const int j = (int)threadIdx.x;
+    const int blocks = PER == 1 ? max(1, 32 / lanes) : 32 * PER;
+    const int bx = (PER == 1 ? q0 / lanes : q0 * PER) + j;
+    if (j >= blocks || bx >= nbx) return;
+    unsigned sum[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        sum[k] = 0u;
+        if (PER == 1) {
+            for (int c = 0; c < min(lanes, 32); ++c) sum[k] += part[k][j * lanes + c];
+        } else {
+            sum[k] = part[8 * (j % PER) + k][j / PER];
+        }
+    }
+    write_cell((long long)by * nbx + bx, sum, counts, rho, ux, uy);
 }
 
 }  // namespace
@@ -93,6 +193,17 @@ cudaError_t launch_coarse_grain(const Geometry& g, const uint32_t* state, const 
                                 bool has_solid, int B, int32_t* counts, float* rho, float* ux,
                                 float* uy, cudaStream_t stream) {
     const int Bw = B / 32, nbx = g.W / B;
+    if (Bw <= 2 || Bw % 4 == 0) {
+        const int per = Bw <= 2 ? 4 / Bw : 1, lanes = Bw <= 2 ? 1 : Bw / 4;   // blocks per quad, quads per block
+        const int width = per > 1 ? 32 : lanes * (lanes >= 32 ? 1 : 32 / lanes);
+        const int groups = (g.Wq + 4 * width - 1) / (4 * width);
+        const unsigned grid = (unsigned)((long long)groups * (g.H / B));
+        auto launch = [&](auto kernel) { kernel<<<grid, kQuadBlock, 0, stream>>>(g, state, solid, B, lanes, groups, counts, rho, ux, uy); };
+        if (per == 4) has_solid ? launch(coarse_quads_kernel<true, 4>) : launch(coarse_quads_kernel<false, 4>);
+        else if (per == 2) has_solid ? launch(coarse_quads_kernel<true, 2>) : launch(coarse_quads_kernel<false, 2>);
+        else has_solid ? launch(coarse_quads_kernel<true, 1>) : launch(coarse_quads_kernel<false, 1>);
+        return cudaGetLastError();
+    }
     const int nb = Bw >= 32 ? 1 : 32 / Bw;
     const int groups = (nbx + nb - 1) / nb;
     const unsigned grid = (unsigned)((long long)groups * (g.H / B));

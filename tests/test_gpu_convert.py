@@ -44,7 +44,7 @@ def test_bytes_and_planes(pkg, W, H, offset):
 
 
 @pytest.mark.parametrize("W,H,B", [(32, 32, 32), (1056, 64, 32), (1152, 192, 96), (960, 320, 160), (2048, 1024, 1024),
-                                   (3072, 1536, 1536), (640, 1280, 640)])
+                                   (3072, 1536, 1536), (640, 1280, 640), (1088, 128, 64), (4096, 4096, 4096), (8448, 128, 128)])
 @pytest.mark.parametrize("solid", [False, True])
 def test_coarse_grain_blocks(pkg, oracle_mod, W, H, B, solid):
     rng = np.random.Generator(np.random.PCG64(W + H + B))
@@ -59,3 +59,22 @@ def test_coarse_grain_blocks(pkg, oracle_mod, W, H, B, solid):
     assert np.array_equal(got[0], want[0])
     for g, r in zip(got[1:], want[1:]):
         np.testing.assert_allclose(g, r.astype(np.float32), rtol=1e-6, atol=1e-30)
+
+
+def test_coarse_grain_sparse_large_block(pkg, oracle_mod):
+    """One block with more fluid nodes than a float counts (2^25 + 2) and few
+    particles: the density is the quotient in doubles, rounded once."""
+    n, mass = 8192, 1001
+    s = np.zeros((n, n), dtype=np.uint8)
+    s[:n // 2] = 0x80
+    s[0, :2] = 0
+    s[n // 2:].reshape(-1)[:mass] = 0x01
+    with pkg.Lattice(n, n, seed=1) as lat:
+        lat.set_state(s)
+        counts, rho, ux, uy = lat.coarse_grain(n)
+    fluid = 2**25 + 2
+    assert counts[0, 0, 7] == fluid and counts[0, 0, 8] == mass
+    assert np.float32(mass / fluid) != np.float32(mass) / np.float32(fluid)
+    assert rho[0, 0] == np.float32(mass / fluid)
+    want = oracle_mod.coarse_grain(s, n)
+    assert ux[0, 0] == np.float32(want[2][0, 0]) and np.isclose(uy[0, 0], want[3][0, 0], rtol=1e-6)
