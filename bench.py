@@ -294,7 +294,7 @@ def batched_vs_per_lattice(dev, stream, count: int, steps: int, per_steps: int, 
             k = b.add(j.W, j.H, j.seed, j.p)
             b.set_state(k, s0)
         # warm-up; the automatic choice times its six candidates here (64 steps each): both kernels at two
-        # tile sizes, and blocked passes of 2 and 4 steps
+        # tile sizes, register marching, and blocked passes of 4 steps
         b.step(384)
         b.synchronize()
         b.step(1)   # reads that measurement
@@ -333,13 +333,14 @@ def batched_vs_per_lattice(dev, stream, count: int, steps: int, per_steps: int, 
         lat.close()
     per = nodes * per_steps / (ms_per / 1e3) / 1e9
     return {"lattices": count, "nodes": nodes, "batched_gsups": batched, "batched_steps": steps,
-            "batched_kernel": ("fhp_batch_block_kernel" if tuned_block > 1 else
+            "batched_kernel": ("fhp_batch_march_kernel" if tuned_block in (2, 3) and not temporal_block else
+                               "fhp_batch_block_kernel" if tuned_block > 1 else
                                "fhp_batch_run_kernel" if tuned == 2 else "fhp_batch_kernel"),
             "batched_tile_quads": tuned_quads,
             "tuned": {"kernel": tuned, "tile_quads": tuned_quads, "temporal_block": tuned_block, "graph_steps": 64,
                       "set_by_flags": bool(step_kernel or temporal_block),
                       "candidates": "single-step graphs / multi-step cooperative x 256 / 128 quads per tile, "
-                                    "and blocked passes of 2 / 4 steps"},
+                                    "register marching (2 or 3 steps), and blocked passes of 4 steps"},
             "batched_launches": launches_batched, "per_lattice_gsups": per, "per_lattice_steps": per_steps,
             "per_lattice_launches": launches_per, "speedup": batched / per,
             "batched_ms": best, "per_lattice_ms": ms_per}
@@ -610,9 +611,10 @@ def run_gpu(args):
     # (steps between hand-offs of strip edge rows), not a blocked pass.
     resident = lat.step_kernel == 4
     if resident and k_block > 1:
-        kernel_name = f"fhp_resident_ghost_kernel (exchange every {k_block} steps)"
+        kernel_name = f"fhp_resident_kernel (exchange every {k_block} steps)"
     elif k_block > 1:
-        kernel_name = f"{'fhp_wave_kernel' if lat.temporal_block_kernel == 1 else 'fhp_block_kernel'} (k={k_block})"
+        blocked = {1: "fhp_wave_kernel", 3: "fhp_march_kernel"}.get(lat.temporal_block_kernel, "fhp_block_kernel")
+        kernel_name = f"{blocked} (k={k_block})"
     k_pass = 1 if resident else k_block
     total_ms = sum(s.elapsed_time(e) for s, e in zip(starts, ends))
     step_kernel_ms = sum(a.elapsed_time(b) for evs in step_ev for a, b in evs)
@@ -626,7 +628,7 @@ def run_gpu(args):
     bytes_per_node = (14 + (1 if has_solid else 0)) / 8.0
     # Step-kernel launches in the timed region: one per lattice step for the
     # single-step kernels, one per fhp_step call (chunks of 2^24 steps) for
-    # the multi-step kernel.
+    # the multi-step kernel and register marching.
     cg_launches = args.steps * chunks if B else 0
     step_launches = max(1, launches - cg_launches)
     steps_per_launch = nsteps * args.steps / step_launches
@@ -746,7 +748,7 @@ def temporal_block_sweep(job, s0, seed, dev, stream, nsteps, peak):
     import torch
     from paper_1208_2428_gb300 import Lattice
     bytes_per_node = (14 + (1 if (s0 & 0x80).any() else 0)) / 8.0
-    names = {0: None, 1: "fhp_wave_kernel", 2: "fhp_block_kernel"}
+    names = {0: None, 1: "fhp_wave_kernel", 2: "fhp_block_kernel", 3: "fhp_march_kernel"}
     out, ref = {}, None
     for k, bk in ((1, 0), (2, 0), (4, 0), (8, 0), (2, 1), (3, 1), (4, 1)):
         with Lattice(job.W, job.H, seed=seed, forcing_p=job.p, device=dev, stream=stream) as lat:
@@ -806,8 +808,10 @@ def rule_set_comparison(job, s0, seed, dev, stream, nsteps, peak):
             e1.record(stream)
             lat.synchronize()
             ms = e0.elapsed_time(e1)
+            marches = lat.temporal_block_kernel == 3
         gsups = job.W * job.H * nsteps / (ms / 1e3) / 1e9
-        out[f"FHP-{'I' * rules}"] = {"gsups": gsups, "ms": ms, "kernel": names.get(kernel, str(kernel)),
+        out[f"FHP-{'I' * rules}"] = {"gsups": gsups, "ms": ms,
+                                     "kernel": "fhp_march_kernel" if marches else names.get(kernel, str(kernel)),
                                      "temporal_block": k,
                                      "hbm_frac": gsups * 1e9 * bytes_per_node / k / (peak * 1e9)}
     return out
