@@ -14,11 +14,14 @@
 // column, so every load is one row segment of a plane.  Where blocks and quads
 // of four words fit each other (1, 2 or a multiple of 4 words per block) a
 // lane's column is a quad and a load of a warp 512 bytes; else it is a word.
-// The latency of the loads bounds it, so 16 warps take two rows at a time:
-// 16384 x 4096, B = 64 (call and flushed caches): 15.3 us; 23.5 us with 8 warps
-// and one row at a time
-// (and with words); 49 us when one warp gathered the words of one block.
-// Repeated, in L2: B = 32 12.5 us, 64 8.4, 128 10.3, 256 14.4.
+// The latency of the loads bounds it, so 16 warps take two rows at a time, and
+// clusters share the rows of large blocks.  16384 x 4096, B = 64, from HBM:
+// 15.3 us; 23.5 us with 8 warps and one row at a time (and with words); 49 us
+// when one warp gathered the words of one block.  Repeated, in L2: B = 32 12.5
+// us, 64 8.4, 128 and more 10.4 (256 14.4 and 512 20.6 without clusters); 4096 x
+// 4096, B = 128 and more: 8.3 (10.3, 14.2, 20.6).
+#include <cooperative_groups.h>
+
 #include "fhp_internal.h"
 
 namespace fhp {
@@ -106,17 +109,22 @@ __global__ void __launch_bounds__(kBlock) coarse_kernel(Geometry g, const uint32
 }
 
 // Quads: a lane counts PER blocks of its four words (4, 2 or 1); `lanes` lanes
-// hold one block where PER is 1.
-template <bool SOLID, int PER>
+// hold one block where PER is 1.  CLUSTER: the `ctas` CTAs of a cluster share the
+// rows of their blocks, B a multiple of 32 * ctas, and add their counts up in the
+// first one's shared memory.
+template <bool SOLID, int PER, bool CLUSTER = false>
 __global__ void __launch_bounds__(kQuadBlock, 2) coarse_quads_kernel(Geometry g, const uint32_t* __restrict__ state,
                                                               const uint32_t* __restrict__ solid, int B, int lanes,
-                                                              int groups, int32_t* __restrict__ counts,
+                                                              int groups, int ctas, int32_t* __restrict__ counts,
                                                               float* __restrict__ rho, float* __restrict__ ux,
                                                               float* __restrict__ uy) {
     __shared__ unsigned part[8 * PER][32 + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nbx = g.W / B;
-    const int by = (int)(blockIdx.x / (unsigned)groups), group = (int)(blockIdx.x - (unsigned)by * (unsigned)groups);
+    if (!CLUSTER) ctas = 1;
+    const unsigned tile = blockIdx.x / (unsigned)ctas;
+    const int rank = CLUSTER ? (int)(blockIdx.x - tile * (unsigned)ctas) : 0;
+    const int by = (int)(tile / (unsigned)groups), group = (int)(tile - (unsigned)by * (unsigned)groups);
     const int width = PER == 1 ? lanes * max(1, 32 / lanes) : 32;   // quads of the CTA
     const int q0 = group * width, quads = min(width, g.nq - q0);
     unsigned n[PER][8];
@@ -142,11 +150,12 @@ __global__ void __launch_bounds__(kQuadBlock, 2) coarse_quads_kernel(Geometry g,
         // (B is a multiple of 32 and a warp takes every 16th row: pairs of rows
         // where the counters leave the registers for it.)
         constexpr int ROWS = PER == 4 ? 1 : 2;
-        for (int r = warp; r < B; r += ROWS * kQuadWarps) {
+        const int stride = ctas * kQuadWarps;
+        for (int r = rank * kQuadWarps + warp; r < B; r += ROWS * stride) {
             uint4 p[ROWS][7], f[ROWS];
 #pragma unroll
             for (int h = 0; h < ROWS; ++h) {
-                const size_t off = base + (size_t)(r + h * kQuadWarps) * g.Pq;
+                const size_t off = base + (size_t)(r + h * stride) * g.Pq;
                 f[h] = SOLID ? *reinterpret_cast<const uint4*>(solid + off) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                 for (int k = 0; k < 7; ++k)
@@ -168,7 +177,18 @@ __global__ void __launch_bounds__(kQuadBlock, 2) coarse_quads_kernel(Geometry g,
     for (int b = 0; b < PER; ++b)
 #pragma unroll
         for (int k = 0; k < 8; ++k) atomicAdd(&part[8 * b + k][lane], n[b][k]);
-    __syncthreads();
+    if (CLUSTER) {
+        auto cluster = cooperative_groups::this_cluster();
+        cluster.sync();
+        if (rank) {
+            unsigned* first = cluster.map_shared_rank(&part[0][0], 0);
+            for (int i = threadIdx.x; i < 8 * PER * 33; i += kQuadBlock) atomicAdd(first + i, part[i / 33][i % 33]);
+        }
+        cluster.sync();
+        if (rank) return;
+    } else {
+        __syncthreads();
+    }
     // Thread j writes block j of the CTA.
     const int j = (int)threadIdx.x;
     const int blocks = PER == 1 ? max(1, 32 / lanes) : 32 * PER;
@@ -198,7 +218,31 @@ cudaError_t launch_coarse_grain(const Geometry& g, const uint32_t* state, const 
         const int width = per > 1 ? 32 : lanes * (lanes >= 32 ? 1 : 32 / lanes);
         const int groups = (g.Wq + 4 * width - 1) / (4 * width);
         const unsigned grid = (unsigned)((long long)groups * (g.H / B));
-        auto launch = [&](auto kernel) { kernel<<<grid, kQuadBlock, 0, stream>>>(g, state, solid, B, lanes, groups, counts, rho, ux, uy); };
+        // Blocks of 128 nodes and more leave few CTAs with many rows each: while no
+        // more than two per SM come of it, the CTAs of a cluster share the rows.  Not
+        // for 32 and 64 nodes, whose few rows gain less than a cluster costs (4096 x
+        // 4096: 8.2 us with, 6.3 without).
+        int ctas = 1;
+        while (per == 1 && ctas < 8 && grid * ctas * 2 <= 304u && B % (64 * ctas) == 0) ctas *= 2;
+        if (ctas > 1) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(grid * ctas);
+            cfg.blockDim = dim3(kQuadBlock);
+            cfg.stream = stream;
+            cudaLaunchAttribute cluster = {};
+            cluster.id = cudaLaunchAttributeClusterDimension;
+            cluster.val.clusterDim.x = ctas;
+            cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+            cfg.attrs = &cluster;
+            cfg.numAttrs = 1;
+            return has_solid ? cudaLaunchKernelEx(&cfg, coarse_quads_kernel<true, 1, true>, g, state, solid, B, lanes,
+                                                  groups, ctas, counts, rho, ux, uy)
+                             : cudaLaunchKernelEx(&cfg, coarse_quads_kernel<false, 1, true>, g, state, solid, B, lanes,
+                                                  groups, ctas, counts, rho, ux, uy);
+        }
+        auto launch = [&](auto kernel) {
+            kernel<<<grid, kQuadBlock, 0, stream>>>(g, state, solid, B, lanes, groups, 1, counts, rho, ux, uy);
+        };
         if (per == 4) has_solid ? launch(coarse_quads_kernel<true, 4>) : launch(coarse_quads_kernel<false, 4>);
         else if (per == 2) has_solid ? launch(coarse_quads_kernel<true, 2>) : launch(coarse_quads_kernel<false, 2>);
         else has_solid ? launch(coarse_quads_kernel<true, 1>) : launch(coarse_quads_kernel<false, 1>);

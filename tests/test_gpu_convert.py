@@ -44,7 +44,8 @@ def test_bytes_and_planes(pkg, W, H, offset):
 
 
 @pytest.mark.parametrize("W,H,B", [(32, 32, 32), (1056, 64, 32), (1152, 192, 96), (960, 320, 160), (2048, 1024, 1024),
-                                   (3072, 1536, 1536), (640, 1280, 640), (1088, 128, 64), (4096, 4096, 4096), (8448, 128, 128)])
+                                   (3072, 1536, 1536), (640, 1280, 640), (1088, 128, 64), (4096, 4096, 4096), (8448, 128, 128),
+                                   (640, 384, 128)])
 @pytest.mark.parametrize("solid", [False, True])
 def test_coarse_grain_blocks(pkg, oracle_mod, W, H, B, solid):
     rng = np.random.Generator(np.random.PCG64(W + H + B))
