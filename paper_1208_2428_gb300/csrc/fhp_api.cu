@@ -551,7 +551,7 @@ int fhp_step(fhp_lattice* h, int64_t n) {
                                                  h->flags + 1);
             if (e != cudaSuccess) return cuda_fail(h, e, "launching the resident kernel");
             ++h->launches;
-            h->cur ^= (chunk & 1);
+            if (fhp::resident_flips(chunk, gh)) h->cur ^= 1;
             h->t += chunk;
             left -= chunk;
         }

@@ -116,11 +116,16 @@ cudaError_t launch_run(const Geometry& g, uint32_t* buf0, uint32_t* buf1, const 
 // steps between exchanges (1, 2 or 4), of which every strip computes gh ghost
 // rows per side itself.  Supported when the strips fit in shared memory and the
 // exchange fits `staging_bytes` of scratch (the lattice's byte-staging area).
-// n >= 1 steps from buf0 (state at t0); the result is in buf0 if n is even,
-// else in buf1.
+// n >= 1 steps from buf0 (state at t0); the result is in buf1 if
+// resident_flips(n, gh), else in buf0.
 bool resident_supported(const Geometry& g, bool has_solid, size_t staging_bytes, int gh = 1);
 // The interval expected to be fastest (0: not supported).
 int resident_interval_for(const Geometry& g, bool has_solid, size_t staging_bytes, bool force);
+// Every strip loads its own rows and its neighbours' edge rows from buf0.  Only
+// the first exchange of edge rows, after step gh, tells a strip that its
+// neighbours have done so: a call of up to gh steps has none, and must not
+// store into buf0 what a strip that starts late has yet to load.
+constexpr bool resident_flips(int nsteps, int gh) { return nsteps % 2 != 0 || nsteps <= gh; }
 cudaError_t launch_resident(const Geometry& g, uint32_t* buf0, uint32_t* buf1, const uint32_t* solid, bool has_solid,
                             bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int nsteps, int gh,
                             uint32_t* halo, size_t halo_bytes, cudaStream_t stream, unsigned int* err);
