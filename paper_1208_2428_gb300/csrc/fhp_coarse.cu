@@ -56,7 +56,7 @@ __device__ __forceinline__ void write_cell(long long cell, const unsigned (&n)[8
         return;
     }
     rho[cell] = __double2float_rn(n[7] ? (double)mass / (double)n[7] : 0.0);
-    ux[cell] = __double2float_rn((double)jx2 / (2.0 * (double)mass));
+    ux[cell] = __double2float_rn(mass ? (double)jx2 / (2.0 * (double)mass) : 0.0);
 }
 
 // Bw words per block row, nb blocks per CTA (nb * Bw <= 32, or nb = 1).

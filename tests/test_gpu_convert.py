@@ -79,3 +79,15 @@ def test_coarse_grain_sparse_large_block(pkg, oracle_mod):
     assert rho[0, 0] == np.float32(mass / fluid)
     want = oracle_mod.coarse_grain(s, n)
     assert ux[0, 0] == np.float32(want[2][0, 0]) and np.isclose(uy[0, 0], want[3][0, 0], rtol=1e-6)
+
+
+@pytest.mark.parametrize("n,solid_rows", [(8192, 0), (8192, 4094), (4096, 0)])
+def test_coarse_grain_empty_large_block(pkg, n, solid_rows):
+    """A block without particles, with 2^26, a little over 2^25 and 2^24 fluid
+    nodes: every field is zero."""
+    with pkg.Lattice(n, n, seed=1) as lat:
+        if solid_rows:
+            lat.load_obstacle_shapes([(pkg.SHAPE_ROWS, 0, solid_rows, 0)])
+        counts, rho, ux, uy = lat.coarse_grain(n)
+    assert counts.reshape(-1).tolist() == [0] * 7 + [n * (n - solid_rows), 0]
+    assert rho[0, 0] == 0.0 and ux[0, 0] == 0.0 and uy[0, 0] == 0.0
