@@ -505,6 +505,8 @@ FHP_API int fhp_batch_coarse_grain(fhp_batch* batch, int32_t slot, int32_t block
 /* Wait for queued work; FHP_ETIMEOUT if a batch kernel gave up waiting. */
 FHP_API int fhp_batch_synchronize(fhp_batch* batch);
 FHP_API int32_t fhp_batch_count(const fhp_batch* batch);
+/* Bytes of the arena not in use (what register marching gives up to any other
+ * use counts as free). */
 FHP_API size_t fhp_batch_free_bytes(const fhp_batch* batch);
 FHP_API int64_t fhp_batch_kernel_launches(const fhp_batch* batch);
 

@@ -1870,7 +1870,10 @@ int32_t fhp_batch_count(const fhp_batch* b) {
     return n;
 }
 
-size_t fhp_batch_free_bytes(const fhp_batch* b) { return b ? b->arena.free_bytes() : 0; }
+// (The counters of register marching are free: take() gives them up.)
+size_t fhp_batch_free_bytes(const fhp_batch* b) {
+    return b ? b->arena.free_bytes() + (b->d_march_flags ? fhp::Arena::round(kMarchFlagBytes) : 0) : 0;
+}
 
 int64_t fhp_batch_kernel_launches(const fhp_batch* b) { return b ? b->launches : -1; }
 

@@ -396,3 +396,34 @@ def test_automatic_choice_without_room_for_blocked_tables(pkg, oracle_mod):
         b.remove(fillers[0])                       # room for the read-back staging (W x H bytes)
         want, _ = oracle_mod.run(s0, job.seed, 0, 98, job.p)
         assert np.array_equal(b.get_state(k), want)
+
+
+def test_free_bytes_counts_what_marching_gives_up(pkg, oracle_mod):
+    """The pass counters of register marching, which any other use of the arena
+    takes back, are free bytes: a caller that compares them with a lattice's
+    size before adding it is not held off by a batch that has marched."""
+    W, H = 256, 128
+    need = pkg.Batch.lattice_bytes(W, H)
+    with pkg.Batch(8 * need) as b:
+        b.add(W, H, 1, 0.0)
+        b.step(1)
+        tight = 8 * need - b.free_bytes + need + 4096      # room for a second member, not for the counters too
+    with pkg.Batch(tight) as b:
+        first = b.add(W, H, 1, 0.0)
+        b.init_random(first, 0.3)
+        b.step(1)
+        before = b.free_bytes
+        assert need <= before <= need + 4096
+        launches = b.kernel_launches
+        b.step(8)
+        assert b.kernel_launches - launches < 8            # it marched
+        assert b.free_bytes == before
+        second = b.add(W, H, 2, 0.0)
+        b.init_random(second, 0.2)
+        assert b.free_bytes == before - need
+        b.step(8)
+        b.synchronize()
+        for slot, seed, rho, n in ((first, 1, 0.3, 17), (second, 2, 0.2, 8)):
+            want, _ = oracle_mod.run(oracle_mod.init_random(W, H, seed, rho), seed, 0, n, 0.0)
+            got = b.coarse_grain_finish(b.coarse_grain_begin(slot, 32))     # (get_state has no room for its bytes)
+            assert np.array_equal(got[0], oracle_mod.coarse_grain(want, 32)[0])
