@@ -271,8 +271,9 @@ FHP_API int fhp_autotune(fhp_lattice* lattice, int32_t trial_steps, int32_t* out
 
 /* Diagnostic: n steps (a multiple of k) as passes of k = 2 or 3 steps by
  * register marching, the kernel the automatic choice uses on large lattices
- * (see fhp_set_step_kernel), on a lattice of any size with H >= 2k + 2;
- * FHP_EINVAL otherwise.  Results are those of fhp_step. */
+ * (see fhp_set_step_kernel), on a lattice of any size with H >= 2k + 2 and rows
+ * that the device's resident warps hold (7.0 million nodes for k = 3, 9.3 million
+ * for k = 2 on GB300); FHP_EINVAL otherwise.  Results are those of fhp_step. */
 FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
 
 /* Step kernel used by fhp_step: 0 = automatic (default), 4 = shared-memory

@@ -187,7 +187,7 @@ void effective_settings(const fhp_lattice* h, int* kernel, int* k_block, int* bk
         if (bk) *bk = kAutoInterval;
         return;
     }
-    if (const int mk = fhp::march_choice(h->g, h->ft, h->force)) {
+    if (const int mk = fhp::march_choice(h->g, h->ft, h->has_solid, h->force)) {
         *k_block = mk;
         if (bk) *bk = 3;
     }
@@ -225,7 +225,7 @@ int resident_interval(const fhp_lattice* h, int kernel, int k_block, int bk) {
 // leave most warps waiting.
 int blocked_kind(const fhp_lattice* h, int k, int bk) {
     if (k <= 1) return 0;
-    if (bk == 3) return fhp::march_supported(h->g, k) ? 3 : 0;
+    if (bk == 3) return fhp::march_fits(h->g, k, h->has_solid, h->force) ? 3 : 0;
     const bool wave = fhp::wave_supported(h->g, k), tiles = fhp::block_supported(h->g, k);
     if (bk == 1) return wave ? 1 : (tiles ? 2 : 0);
     return tiles ? 2 : (wave ? 1 : 0);
@@ -516,9 +516,9 @@ int march_steps(fhp_lattice* h, int k, int64_t* n) {
 int fhp_step_march(fhp_lattice* h, int32_t k, int64_t n) {
     if (!h) return fail(nullptr, FHP_EINVAL, "lattice is NULL");
     if (n < 0 || n > kMaxTime - h->t) return fail(h, FHP_EINVAL, "step count %lld out of range", (long long)n);
-    if ((k != 2 && k != 3) || n % k || !fhp::march_supported(h->g, k))
-        return fail(h, FHP_EINVAL, "passes of %d steps do not cover %lld steps of this lattice", k, (long long)n);
     DeviceGuard dg(h->device);
+    if ((k != 2 && k != 3) || n % k || !fhp::march_fits(h->g, k, h->has_solid, h->force))
+        return fail(h, FHP_EINVAL, "passes of %d steps do not cover %lld steps of this lattice", k, (long long)n);
     return march_steps(h, k, &n);
 }
 
@@ -744,6 +744,7 @@ int fhp_set_rows_device(fhp_lattice* h, int32_t y0, int32_t n, const uint32_t* d
 
 int fhp_get_temporal_block(const fhp_lattice* h) {
     if (!h) return -1;
+    DeviceGuard dg(h->device);
     int kernel, k_block, bk;
     effective_settings(h, &kernel, &k_block, &bk);
     const int gh = resident_interval(h, kernel, k_block, bk);
@@ -760,6 +761,7 @@ int fhp_set_temporal_block_kernel(fhp_lattice* h, int32_t kind) {
 
 int fhp_get_temporal_block_kernel(const fhp_lattice* h) {
     if (!h) return -1;
+    DeviceGuard dg(h->device);
     int kernel, k_block, bk;
     effective_settings(h, &kernel, &k_block, &bk);
     if (resident_interval(h, kernel, k_block, bk) > 0) return 0;
@@ -806,8 +808,8 @@ int fhp_autotune(fhp_lattice* h, int32_t trial_steps, int32_t* out_kernel, int32
         if (fhp::block_supported(h->g, k)) cands.push_back({fhp::kStepDirect, k, 2});
     // Register marching (remainders on the ring kernel where a row fits it).
     const int rest_kernel = fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepRing);
-    const int mk = fhp::march_choice(h->g, h->ft, h->force);
-    if (mk == 2 || (h->g.rules != 3 && fhp::march_supported(h->g, 2))) cands.push_back({rest_kernel, 2, 3});
+    const int mk = fhp::march_choice(h->g, h->ft, h->has_solid, h->force);
+    if (mk == 2 || (h->g.rules != 3 && fhp::march_fits(h->g, 2, h->has_solid, h->force))) cands.push_back({rest_kernel, 2, 3});
     if (mk == 3) cands.push_back({rest_kernel, 3, 3});
     TuneChoice best{fhp::kStepDirect, 1, 0};
     float best_ms = -1.0f;

@@ -183,9 +183,13 @@ cudaError_t launch_wave(const Geometry& g, const uint32_t* src, uint32_t* dst, c
 // `flags` is scratch of `flag_bytes` (a word per warp; too few: one launch per
 // pass).
 bool march_supported(const Geometry& g, int k);
+// ... and whether one resident wave of the current device's warps holds a
+// band's columns (rows of up to 7.0 million nodes for k = 3, 9.3 million for k =
+// 2 on 152 SMs), without which launch_march refuses.
+bool march_fits(const Geometry& g, int k, bool has_solid, bool force);
 // Steps per pass for which register marching is the automatic choice (0: it
 // is not).
-int march_choice(const Geometry& g, const ForcingTable& ft, bool force);
+int march_choice(const Geometry& g, const ForcingTable& ft, bool has_solid, bool force);
 cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const uint32_t* solid, bool has_solid,
                          bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int k, int passes,
                          unsigned int* flags, size_t flag_bytes, cudaStream_t stream, unsigned int* err);

@@ -24,6 +24,19 @@ cudaError_t march_any(int k, const StepArgs& a, const MarchArgs& b, const MarchV
     return k == 2 ? march_k<2>(a, b, v, launch, n, s) : march_k<3>(a, b, v, launch, n, s);
 }
 
+MarchVariant march_variant_of(const Geometry& g, bool has_solid, bool force) {
+    return MarchVariant{has_solid, force, g.Wq % 4 != 0, g.rules == 3};
+}
+
+// Warps of the variant's kernel that are resident at once.
+cudaError_t march_resident(int k, const MarchVariant& v, int* warps) {
+    int per_sm = 0;
+    const cudaError_t e = march_any(k, StepArgs{}, MarchArgs{}, v, false, &per_sm, nullptr);
+    if (e != cudaSuccess) return e;
+    *warps = march_sms() * per_sm * kMarchWarps;
+    return *warps > 0 ? cudaSuccess : cudaErrorInvalidDevice;
+}
+
 }  // namespace
 
 // How the quad columns of a lattice's bands go to lanes.  Rows of few quads:
@@ -81,6 +94,13 @@ bool march_supported(const Geometry& g, int k) {
     return (k == 2 || k == 3) && g.H >= 2 * k + 2 && g.plane_words * 4 < ((size_t)1 << 32) - 64;
 }
 
+bool march_fits(const Geometry& g, int k, bool has_solid, bool force) {
+    int resident = 0;
+    return march_supported(g, k) &&
+           march_resident(k, march_variant_of(g, has_solid, force), &resident) == cudaSuccess &&
+           march_warps(g, march_layout(g, k), g.H) <= resident;
+}
+
 // Where register marching is the automatic choice (GB300, GSUPS, marching
 // against the kernel it replaces; the lattices hold a cylinder):
 //   without forcing   8192 x 2560: 3.8 thousand with k = 2 (3.7 with k = 3)
@@ -95,15 +115,17 @@ bool march_supported(const Geometry& g, int k) {
 //     with p: 3.7 against 3.6 at p = 2e-3, 3.6 against 3.6 at 4e-3;
 //   FHP-III   from 200 million nodes on: its network is as long as the memory
 //     traffic it hides on smaller lattices.
-int march_choice(const Geometry& g, const ForcingTable& ft, bool force) {
+int march_choice(const Geometry& g, const ForcingTable& ft, bool has_solid, bool force) {
     if (!march_supported(g, 3)) return 0;
     const long long nodes = (long long)g.W * g.H;
+    int k = 0;
     if (force) {
         const bool rare = ft.p_plus_1 <= (1ull << 32) / 400;   // p < 2.5e-3
-        return rare && nodes >= (g.rules == 3 ? 200000000LL : 40000000LL) ? 2 : 0;
+        if (rare && nodes >= (g.rules == 3 ? 200000000LL : 40000000LL)) k = 2;
+    } else if (nodes >= 12000000) {
+        k = nodes < 48000000 ? 2 : 3;
     }
-    if (nodes < 12000000) return 0;
-    return nodes < 48000000 ? 2 : 3;
+    return k && march_fits(g, k, has_solid, force) ? k : 0;
 }
 
 cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const uint32_t* solid, bool has_solid,
@@ -124,12 +146,10 @@ cudaError_t launch_march(const Geometry& g, uint32_t* src, uint32_t* dst, const 
     a.err = err;
     a.ft = ft;
     MarchArgs b{};
-    const MarchVariant v{has_solid, force, g.Wq % 4 != 0, g.rules == 3};
-    int per_sm = 0;
-    cudaError_t e = march_any(k, a, b, v, false, &per_sm, stream);
+    const MarchVariant v = march_variant_of(g, has_solid, force);
+    int resident = 0;
+    cudaError_t e = march_resident(k, v, &resident);
     if (e != cudaSuccess) return e;
-    const int resident = march_sms() * per_sm * kMarchWarps;
-    if (resident <= 0) return cudaErrorInvalidDevice;
 
     const MarchLayout lay = march_layout(g, k);
     b.pitch = lay.pitch;

@@ -83,6 +83,23 @@ def test_automatic_choice_equals_direct_kernel(pkg, W, H, p, block):
     assert torch.equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("W,p", [(7_200_000, 0.0), (7_200_032, 0.0), (9_600_000, 0.0), (9_600_000, 5e-4)])
+def test_rows_too_wide_to_march(pkg, W, p):
+    """Rows of more columns than the warps of one resident wave hold (7.0 million
+    nodes for passes of 3 steps, 9.3 million for 2 on 152 SMs): the automatic
+    choice steps them with a kernel that can."""
+    import torch
+    H, got = 8, []
+    for kernel in (0, 1):
+        with pkg.Lattice(W, H, seed=5, forcing_p=p, step_kernel=kernel) as lat:
+            lat.load_obstacle_shapes([(pkg.SHAPE_ROWS, 0, 1, 0), (pkg.SHAPE_DISC, W // 2, 4, 2)])
+            lat.init_random(0.3)
+            lat.step(7)
+            got.append(lat.get_state_tensor())
+            lat.synchronize()
+    assert torch.equal(got[0], got[1])
+
+
 def test_march_refusals(pkg):
     with pkg.Lattice(64, 6, seed=1) as lat:
         lat.step_march(2, 0)
