@@ -294,7 +294,8 @@ FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
  * the intermediate time levels in registers, all passes of a call in one
  * cooperative launch, and only a remaining step runs on the kernels below.
  * Else it picks 1 for lattices of fewer than 8 tiles, 3 up to 24 tiles per SM
- * (single steps: 1) and 1 above.
+ * and single steps above (and for what is left over): 2 for lattices beyond L2
+ * whose rows are narrow or leave many lanes of the direct kernel empty, else 1.
  * Results are identical for every choice.  While the kernel is automatic and the temporal block 1, a
  * configuration recorded by fhp_autotune for the lattice's description takes
  * precedence. */

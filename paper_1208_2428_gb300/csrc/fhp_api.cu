@@ -581,7 +581,7 @@ int fhp_step(fhp_lattice* h, int64_t n) {
             n -= k;
         }
     }
-    if (n >= 2 && fhp::resolved_step_kernel(h->g, h->has_solid, kernel) == fhp::kStepRun) {
+    if (n >= 2 && fhp::resolved_step_kernel(h->g, h->has_solid, h->force, kernel) == fhp::kStepRun) {
         // All n steps in cooperative launches of up to 2^24 steps each.
         int64_t left = n;
         while (left > 0) {
@@ -690,8 +690,8 @@ int fhp_get_step_kernel(const fhp_lattice* h) {
     if (kernel == fhp::kStepResident)
         return fhp::resident_supported(h->g, h->has_solid, h->staging_bytes)
                    ? reported_kernel(h, kernel)
-                   : fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepAuto);
-    return fhp::resolved_step_kernel(h->g, h->has_solid, kernel);
+                   : fhp::resolved_step_kernel(h->g, h->has_solid, h->force, fhp::kStepAuto);
+    return fhp::resolved_step_kernel(h->g, h->has_solid, h->force, kernel);
 }
 
 int fhp_set_rules(fhp_lattice* h, int32_t rules) {
@@ -793,7 +793,7 @@ int fhp_autotune(fhp_lattice* h, int32_t trial_steps, int32_t* out_kernel, int32
     if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
     std::vector<TuneChoice> cands;
     cands.push_back({fhp::kStepDirect, 1, 0});
-    if (fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepRing) != fhp::kStepDirect) {
+    if (fhp::resolved_step_kernel(h->g, h->has_solid, h->force, fhp::kStepRing) != fhp::kStepDirect) {
         cands.push_back({fhp::kStepRing, 1, 0});
         cands.push_back({fhp::kStepRun, 1, 0});
     }
@@ -806,8 +806,8 @@ int fhp_autotune(fhp_lattice* h, int32_t trial_steps, int32_t* out_kernel, int32
         if (fhp::wave_supported(h->g, k)) cands.push_back({fhp::kStepDirect, k, 1});
     for (int k : {2, 4, 8})
         if (fhp::block_supported(h->g, k)) cands.push_back({fhp::kStepDirect, k, 2});
-    // Register marching (remainders on the ring kernel where a row fits it).
-    const int rest_kernel = fhp::resolved_step_kernel(h->g, h->has_solid, fhp::kStepRing);
+    // Register marching (remaining steps on the faster kernel of single steps).
+    const int rest_kernel = fhp::single_step_kernel(h->g, h->has_solid, h->force);
     const int mk = fhp::march_choice(h->g, h->ft, h->has_solid, h->force);
     if (mk == 2 || (h->g.rules != 3 && fhp::march_fits(h->g, 2, h->has_solid, h->force))) cands.push_back({rest_kernel, 2, 3});
     if (mk == 3) cands.push_back({rest_kernel, 3, 3});

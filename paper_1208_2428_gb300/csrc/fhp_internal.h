@@ -98,8 +98,12 @@ cudaError_t launch_step(const Geometry& g, const uint32_t* src, uint32_t* dst,
                         unsigned int* err = nullptr, int kernel = kStepAuto);
 
 // The kernel fhp_step uses for `requested`: kStepDirect, kStepRing or kStepRun
-// (launch_step itself runs kStepDirect for kStepRun: one step per launch).
-int resolved_step_kernel(const Geometry& g, bool has_solid, int requested);
+// (launch_step itself runs single_step_kernel's for kStepRun: one step per
+// launch).
+int resolved_step_kernel(const Geometry& g, bool has_solid, bool force, int requested);
+
+// The faster kernel of single steps: kStepDirect or kStepRing.
+int single_step_kernel(const Geometry& g, bool has_solid, bool force);
 
 // Tiles of the ring / multi-step kernels (0 if a row does not fit a stage);
 // the multi-step kernel needs that many counter words of scratch.

@@ -23,7 +23,7 @@
 //                          tiles are in flight while 8 consumer warps compute;
 //   fhp_step_direct_kernel one quad per thread, operands loaded straight into
 //                          registers and neighbour words exchanged with
-//                          __shfl_sync (the automatic choice for single steps).
+//                          __shfl_sync (single steps, except where single_step_kernel says).
 #include <cstdio>
 #include <mutex>
 
@@ -543,7 +543,33 @@ Geometry make_geometry(int W, int H) {
     return g;
 }
 
-int resolved_step_kernel(const Geometry& g, bool has_solid, int requested) {
+// The kernel of a single step.  The direct kernel streams best where its warps
+// are full and their loads contiguous, with 32 warps an SM against the ring's 18
+// (time of a ring step over a direct one, p = 0 / 5e-4 / 0.02, 134 million nodes:
+// rows of 128 quads 1.10 / 1.11 / 1.09, 32 quads 1.11 / 1.12 / 1.10, 8 quads 1.16
+// / 1.15 / 1.12; FHP-III 1.06; 8192 x 4096 1.25 / 1.16 / 1.09).  Beyond L2 the
+// ring, whose tiles are whole rows however the quads fall on lanes, wins
+//   for rows of fewer than 16 quads, of which a direct warp takes several, every
+//     second one of the lattice: 1 quad 0.48 / 0.49 / 0.49, 2 0.71 / 0.71 / 0.71, 3
+//     0.44 / 0.46 / 0.46, 7 0.50, 9 0.57, 12 0.93 / 0.92 / 0.86 (but 8 quads,
+//     aligned with the lanes and the memory's sectors).  At 67 million padded
+//     nodes 0.50 to 0.88, at 40 million about 1;
+//   where rows leave over 42 % of the lanes empty: 17 quads 0.77 / 0.75 / 0.64 (24
+//     million nodes 0.98 / 0.77 / 0.74), 33 quads 0.98 / 0.83 / 0.75;
+//   and where they leave 30 % empty, with forcing (20 quads 0.99 / 0.92 / 0.76, 40
+//     quads 1.09 / 0.99 / 0.89), or 25 %, for FHP-III (24 quads 0.84).
+int single_step_kernel(const Geometry& g, bool has_solid, bool force) {
+    if (tile_rows(g, has_solid) == 0) return kStepDirect;
+    const size_t padded = g.plane_words * 32;
+    const int per_warp = g.nq < 32 ? 32 / g.nq : 1, warps = g.nq < 32 ? 1 : (g.nq + 31) / 32;
+    const int used = 1000 * per_warp * g.nq / (32 * warps);   // lanes in use, per mille
+    if (padded >= 20000000 && used <= 580) return kStepRing;
+    if (padded < 50000000) return kStepDirect;
+    const bool narrow = g.nq < 16 && g.nq != 8;
+    return narrow || (force && used <= 700) || (g.rules == 3 && used <= 750) ? kStepRing : kStepDirect;
+}
+
+int resolved_step_kernel(const Geometry& g, bool has_solid, bool force, int requested) {
     const int R = tile_rows(g, has_solid);
     if (R == 0 || requested == kStepDirect) return kStepDirect;
     if (requested == kStepRing || requested == kStepRun) return requested;
@@ -559,14 +585,11 @@ int resolved_step_kernel(const Geometry& g, bool has_solid, int requested) {
     // Few tiles per CTA and step: launch gaps and per-step pipeline refills
     // dominate, so run all steps in one launch (measured on GB300: 984 vs 713
     // GSUPS on 4096 x 1024, 3600 vs 3273 on 16384 x 4096).  Many tiles per CTA:
-    // the per-step overhead is small and the direct kernel streams best, with
-    // 32 warps an SM against the ring's 18: on 29,984 x 27,990 3702 GSUPS (6.9
-    // TB/s of algorithmic bytes) against the ring's 3051, on 16384 x 8192 3372
-    // against 2976 (FHP-III).  A lattice of a handful of tiles is faster with
-    // the direct kernel.
+    // the per-step overhead is small and single steps stream better.  A lattice
+    // of a handful of tiles is faster with the direct kernel.
     const int ntiles = (g.H + R - 1) / R;
     if (ntiles < 8) return kStepDirect;
-    return ntiles <= 12 * 2 * sms ? kStepRun : kStepDirect;
+    return ntiles <= 12 * 2 * sms ? kStepRun : single_step_kernel(g, has_solid, force);
 }
 
 int run_tiles(const Geometry& g, bool has_solid) {
@@ -640,10 +663,9 @@ cudaError_t launch_step(const Geometry& g, const uint32_t* src, uint32_t* dst,
     a.ft = ft;
     const bool ragged = (g.Wq % 4) != 0;
     const int R = tile_rows(g, has_solid);
-    // (A lattice the multi-step kernel would run takes a single step with the
-    // direct kernel: 8192 x 4096 3270 against the ring's 2807 GSUPS, 4096 x 1024
-    // 713 against 681.)
-    if (resolved_step_kernel(g, has_solid, kernel) == kStepRing) {
+    kernel = resolved_step_kernel(g, has_solid, force, kernel);
+    if (kernel == kStepRun) kernel = single_step_kernel(g, has_solid, force);
+    if (kernel == kStepRing) {
         TileArgs ta;
         ta.R = R;
         ta.ntiles = (g.H + R - 1) / R;

@@ -83,6 +83,27 @@ def test_automatic_choice_equals_direct_kernel(pkg, W, H, p, block):
     assert torch.equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("W,H,p,rules", [(32, 400_000, 0.02, 2), (96, 400_000, 0.02, 1), (384, 140_000, 0.02, 2),
+                                         (1152, 45_000, 0.0, 3), (2176, 15_000, 0.02, 2), (4192, 8_000, 0.02, 2),
+                                         (2560, 22_000, 0.02, 2), (3040, 20_000, 0.02, 3), (1024, 60_000, 0.02, 2)])
+def test_single_steps_of_large_lattices_equal_direct_kernel(pkg, W, H, p, rules):
+    """Lattices beyond L2 whose rows are narrow or leave lanes empty (ragged ones
+    among them), on either side of the rule's lines: single steps and calls of
+    several against the direct kernel."""
+    import torch
+    got = []
+    for kernel in (0, 1):
+        with pkg.Lattice(W, H, seed=6, forcing_p=p, step_kernel=kernel) as lat:
+            lat.set_rules(rules)
+            lat.load_obstacle_shapes(workloads.cylinder_shapes(W, H))
+            lat.init_random(0.3)
+            for n in (1, 1, 4):
+                lat.step(n)
+            got.append(lat.get_state_tensor())
+            lat.synchronize()
+    assert torch.equal(got[0], got[1])
+
+
 @pytest.mark.parametrize("W,p", [(7_200_000, 0.0), (7_200_032, 0.0), (9_600_000, 0.0), (9_600_000, 5e-4)])
 def test_rows_too_wide_to_march(pkg, W, p):
     """Rows of more columns than the warps of one resident wave hold (7.0 million
