@@ -289,7 +289,8 @@ FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
  * lattices whose strips fit (calls of up to three steps: 1; FHP-III lattices
  * report it as 3, all steps of a call in one launch), else register marching for lattices of 12 million nodes and more
  * (40 million with forcing, whose probability must be below 0.0025; 200
- * million for forced FHP-III lattices): passes of 2 or 3 steps in which every
+ * million for forced FHP-III lattices; not for lattices beyond L2 of at most
+ * 128 columns): passes of 2 or 3 steps in which every
  * lane of a warp marches a column of 128-node quads up a band of rows with
  * the intermediate time levels in registers, all passes of a call in one
  * cooperative launch, and only a remaining step runs on the kernels below.

@@ -114,16 +114,25 @@ bool march_fits(const Geometry& g, int k, bool has_solid, bool force) {
 //     walks behind instead of 16: 3.2 on 16384 x 4096).  The walk's cost grows
 //     with p: 3.7 against 3.6 at p = 2e-3, 3.6 against 3.6 at 4e-3;
 //   FHP-III   from 200 million nodes on: its network is as long as the memory
-//     traffic it hides on smaller lattices.
+//     traffic it hides on smaller lattices;
+//   rows of one quad (at most 128 nodes)   every lane marches a band of its own and
+//     a warp's loads are 16-byte pieces far apart, each of which costs a whole
+//     sector, so beyond L2 the ring and its contiguous tiles win (time marching
+//     over the faster single-step kernel, by nodes with padding): with k = 3 53
+//     million 0.77 to 0.91, 80 million 0.94, 90 million 1.03 to 1.08, 130 million
+//     1.05 to 1.15, 270 million 1.25 to 1.5; with k = 2 53 million 0.90 to 0.95, 66
+//     million 1.2 to 1.4, 130 million 1.5 to 2 -- so k = 3 below 85 million without
+//     forcing, k = 2 below 60 million with it.
 int march_choice(const Geometry& g, const ForcingTable& ft, bool has_solid, bool force) {
     if (!march_supported(g, 3)) return 0;
     const long long nodes = (long long)g.W * g.H;
     int k = 0;
+    if (g.nq == 1 && g.plane_words * 32 >= (force ? 60000000u : 85000000u)) return 0;
     if (force) {
         const bool rare = ft.p_plus_1 <= (1ull << 32) / 400;   // p < 2.5e-3
         if (rare && nodes >= (g.rules == 3 ? 200000000LL : 40000000LL)) k = 2;
     } else if (nodes >= 12000000) {
-        k = nodes < 48000000 ? 2 : 3;
+        k = nodes < 48000000 && g.nq > 1 ? 2 : 3;
     }
     return k && march_fits(g, k, has_solid, force) ? k : 0;
 }

@@ -121,6 +121,25 @@ def test_rows_too_wide_to_march(pkg, W, p):
     assert torch.equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("W,H,p,block", [(32, 600_000, 0.0, 3), (32, 700_000, 0.0, 0), (128, 400_000, 5e-4, 2),
+                                         (128, 480_000, 5e-4, 0), (96, 500_000, 0.0, 3), (160, 240_000, 0.0, 2)])
+def test_automatic_choice_for_narrow_rows(pkg, W, H, p, block):
+    """Rows of one quad on either side of the lines of the automatic choice (0:
+    they do not march), and rows of two quads, against the direct kernel."""
+    import torch
+    got = []
+    for kernel in (0, 1):
+        with pkg.Lattice(W, H, seed=5, forcing_p=p, step_kernel=kernel) as lat:
+            lat.load_obstacle_shapes(workloads.cylinder_shapes(W, H))
+            lat.init_random(0.3)
+            if kernel == 0:
+                assert (lat.temporal_block_kernel, lat.temporal_block) == ((3, block) if block else (0, 1))
+            lat.step(11)
+            got.append(lat.get_state_tensor())
+            lat.synchronize()
+    assert torch.equal(got[0], got[1])
+
+
 def test_march_refusals(pkg):
     with pkg.Lattice(64, 6, seed=1) as lat:
         lat.step_march(2, 0)
