@@ -286,7 +286,7 @@ FHP_API int fhp_step_march(fhp_lattice* lattice, int32_t k, int64_t n);
  * running all steps of an fhp_step call in one cooperative launch, each tile
  * waiting only for the three tiles of the previous step it reads).  2 and 3
  * fall back to 1 when a row does not fit a stage.  Automatic picks 4 for
- * lattices whose strips fit (calls of up to three steps: 1; FHP-III lattices
+ * lattices whose strips fit (calls of up to three steps, and of up to nine of flat lattices: 1; FHP-III lattices
  * report it as 3, all steps of a call in one launch), else register marching for lattices of 12 million nodes and more
  * (40 million with forcing, whose probability must be below 0.0025; 200
  * million for forced FHP-III lattices; not for lattices beyond L2 of at most

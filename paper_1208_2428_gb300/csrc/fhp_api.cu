@@ -532,9 +532,7 @@ int fhp_step(fhp_lattice* h, int64_t n) {
     int kernel = h->step_kernel, k_block = h->k_block, bk = h->block_kernel;
     effective_settings(h, &kernel, &k_block, &bk);
     int gh = resident_interval(h, kernel, k_block, bk);
-    if (gh > 0 && n <= 3 && h->step_kernel == fhp::kStepAuto) {
-        // Up to three steps do not repay moving the lattice into shared memory
-        // and back (about 10 us; a direct step of such a lattice takes 4 to 6).
+    if (gh > 0 && h->step_kernel == fhp::kStepAuto && n < fhp::resident_least_steps(h->g, h->force)) {
         gh = 0;
         kernel = fhp::kStepDirect;
         k_block = 1;

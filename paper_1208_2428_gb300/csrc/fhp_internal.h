@@ -125,6 +125,9 @@ cudaError_t launch_run(const Geometry& g, uint32_t* buf0, uint32_t* buf1, const 
 bool resident_supported(const Geometry& g, bool has_solid, size_t staging_bytes, int gh = 1);
 // The interval expected to be fastest (0: not supported).
 int resident_interval_for(const Geometry& g, bool has_solid, size_t staging_bytes, bool force);
+// The least number of steps for which moving the lattice into shared memory and
+// back pays (the direct kernel takes shorter calls of the automatic choice).
+int resident_least_steps(const Geometry& g, bool force);
 // Every strip loads its own rows and its neighbours' edge rows from buf0.  Only
 // the first exchange of edge rows, after step gh, tells a strip that its
 // neighbours have done so: a call of up to gh steps has none, and must not

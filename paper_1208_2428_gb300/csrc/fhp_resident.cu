@@ -76,6 +76,20 @@ int resident_interval_for(const Geometry& g, bool has_solid, size_t staging_byte
     return resident_supported(g, has_solid, staging_bytes, 1) ? 1 : 0;
 }
 
+// Moving a lattice in and out costs 8 to 10 us, a direct step 4.15 us while its
+// launch bounds it: calls of up to three steps are direct.  Flat lattices of long
+// rows have fewer strips than SMs, each of two rows, and a step takes longer the
+// longer the rows: 2.0 us for 128 quads, 2.7 for 192, 3.2 for 250 (us a call,
+// resident / direct: 32384 x 4, 4 steps 22.8 / 16.8, 8 steps 35.5 / 33.1, 12 steps
+// 48.5 / 49.5; 24576 x 32, 6 steps 26.7 / 24.9, 8 steps 31.8 / 33.1; 16384 x 32, 4
+// steps 17.3 / 16.7, 5 steps 18.9 / 20.8).  One strip alone has no rows to hand
+// over (32768 x 2, 4 steps 12.8 / 16.7), and a forced direct step of more than 2
+// million nodes takes longer than its launch (32768 x 152, 5 steps 28.9 / 30.5).
+int resident_least_steps(const Geometry& g, bool force) {
+    const bool flat = g.H >= 4 && g.H < 2 * resident_sms() && !(force && (long long)g.W * g.H > 2000000);
+    return std::max(4, flat ? g.nq / 28 + 1 : 0);
+}
+
 cudaError_t launch_resident(const Geometry& g, uint32_t* buf0, uint32_t* buf1, const uint32_t* solid, bool has_solid,
                             bool force, const ForcingTable& ft, Key2 key, uint64_t t0, int nsteps, int gh,
                             uint32_t* halo, size_t halo_bytes, cudaStream_t stream, unsigned int* err) {

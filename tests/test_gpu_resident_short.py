@@ -44,3 +44,18 @@ def test_calls_without_an_exchange(pkg, oracle_mod, W, H, interval, n, p):
     assert t == 7 * n + 1
     want, _ = oracle_mod.run(s0, seed, 0, t, p)
     assert np.array_equal(got, want), f"{int((got != want).sum())} nodes differ"
+
+
+@pytest.mark.parametrize("W,H,p", [(32384, 4, 0.0), (24608, 6, 0.02), (16384, 32, 0.0), (32768, 2, 0.02), (1024, 8, 0.0)])
+def test_short_calls_of_flat_lattices(pkg, oracle_mod, W, H, p):
+    """Calls on either side of the number of steps from which the automatic
+    choice keeps a flat lattice in shared memory."""
+    seed = W + H
+    s0 = workloads.bernoulli_lattice(W, H, 0.3, seed, workloads.channel_walls(W, H) if p and H > 2 else None)
+    with pkg.Lattice(W, H, seed=seed, forcing_p=p) as lat:
+        lat.set_state(s0)
+        for n in range(3, 13):
+            lat.step(n)
+        got = lat.get_state()
+    want, _ = oracle_mod.run(s0, seed, 0, sum(range(3, 13)), p)
+    assert np.array_equal(got, want), f"{int((got != want).sum())} nodes differ"
