@@ -423,7 +423,8 @@ FHP_API int fhp_batch_step(fhp_batch* batch, int64_t n);
  * capture, device tables, kernel attributes), and a later call records the
  * candidate with the most node updates per millisecond for the class (read
  * without waiting); until then, while the temporal block is automatic too,
- * register marching runs (see fhp_batch_set_temporal_block), else
+ * register marching runs (see fhp_batch_set_temporal_block) where the sizes and
+ * forcing of the members and the length of the call let it pay, else
  * SINGLE_STEP with 256-quad tiles and no blocking.  Results are identical for
  * every choice. */
 #define FHP_BATCH_KERNEL_AUTO 0

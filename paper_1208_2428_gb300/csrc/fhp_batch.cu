@@ -1449,6 +1449,58 @@ int march_block(const fhp_batch* b) {
     return march_split(plain, forced) ? march_block_for(plain, false) : march_block_for(plain + forced, forced > 0);
 }
 
+// Whether a call of n steps of a batch that has not been tuned marches (times of
+// marching over single steps of the whole batch):
+//   every member marches, up to 256 of them: 0.35 to 0.9 -- but 3 or 5 steps in
+//     passes of 2 end in a single one, for which every member's descriptors go up:
+//     0.9 with 64 members, 1.08 with 150, 1.17 with 256 (5 steps: 1.0);
+//   several groups of 256, one launch after the other, each of which takes about
+//     9 us a pass however small its members: 300 x 64 x 32 0.7 to 0.9, but 1.32
+//     from graph_steps on, where single steps come from the graph; 1000 x 64 x 32
+//     1.20 for 2 steps, 0.95 for 8.  From 8 million nodes a group on without
+//     forcing (300 x 256 x 256 0.63 to 0.85; from four groups on 12 million, 1000 x
+//     256 x 128 having 0.83 to 1.14) and 25 million with it (600 x 512 x 256 0.82
+//     to 0.92; 600 x 256 x 256 1.06 to 1.14) it always pays;
+//   members that do not march need launches of their own for every step, 4 us each
+//     (rows too few: 128 million nodes beside one such member 0.6 to 0.8, 0.8 to
+//     0.95 with forcing) or 10 to 17 us (dense forcing: beside one of 1024 x 1024 15
+//     million nodes 1.3 to 1.6, 95 million 1.0 to 1.4, 170 million without forcing
+//     and 5 steps or more 0.9 to 0.98, 670 million with forcing 1.1);
+//   one quad column: marching is slow beyond L2 (march_choice; 63 x 64 x 16384 1.3
+//     to 1.8 with forcing, without it 1.6 for 4 steps and, in passes of 3, 0.88 for
+//     32).
+bool march_pays(const fhp_batch* b, int n) {
+    long long plain = 0, forced = 0, padded = 0, narrow = 0;
+    int count = 0;
+    bool rest = false, dense = false;
+    for (const Member& m : b->members) {
+        if (!m.used || m.steps_left == 0) continue;
+        const bool force = m.ft.q[32] != 0;
+        if (!marches(m, 2)) {
+            rest = true;
+            dense = dense || force;
+            continue;
+        }
+        ++count;
+        (force ? forced : plain) += (long long)m.g.W * m.g.H;
+        const long long p = (long long)m.g.plane_words * 32;
+        padded += p;
+        if (m.g.nq == 1) narrow += p;
+    }
+    if (count == 0 || n < 2) return false;
+    if (rest) {
+        if (dense) return forced == 0 && plain >= 150000000 && n >= 5;
+        return plain + forced >= (forced ? 100000000 : 40000000);
+    }
+    const int k = march_split(plain, forced) ? 2 : march_block_for(plain + forced, forced > 0);
+    if (narrow >= 60000000 && 2 * narrow >= padded) return k == 3 && narrow < 200000000 && n >= 16;
+    if (k == 2 && (n == 3 || n == 5) && count > 128) return false;
+    const int groups = (count + fhp::kMarchJobs - 1) / fhp::kMarchJobs;
+    if (groups == 1 || (plain + forced) / groups >= (forced ? 25000000 : groups <= 3 ? 8000000 : 12000000)) return true;
+    const bool graph = b->graph_steps > 0 && n >= b->graph_steps;
+    return !graph && (forced ? groups == 2 : groups <= 3 || n >= 5);
+}
+
 // One cooperative launch per group of members: member i advances by
 // passes[i] passes of k steps.
 int launch_march_passes(fhp_batch* b, int k, const std::vector<int>& passes) {
@@ -1751,7 +1803,7 @@ int batch_step(fhp_batch* b, int64_t n) {
                 k = b->tuned_block[cls];
                 march = b->tuned_march[cls];
             } else {
-                march = chunk >= 2 && reserve_march(b);
+                march = march_pays(b, chunk) && reserve_march(b);
             }
             march = march && march_block(b) != 0;   // (the members may have changed since the trial)
             if (!march && b->tuned_march[cls]) k = 1;

@@ -195,3 +195,51 @@ def test_batch_of_more_members_than_a_launch_holds(pkg, oracle_mod):
             w, h, seed, rho = jobs[i]
             want, _ = oracle_mod.run(oracle_mod.init_random(w, h, seed, rho), seed, 0, 6, 0.0)
             assert np.array_equal(b.get_state(slots[i]), want), i
+
+
+def _mixed(kind):
+    """Members beside which an untuned batch marches, or does not."""
+    big = [(2048, 2048, 0.0)] * 10
+    return {"all": [(512, 384, 0.0)] * 6,
+            "one dense": [(512, 384, 0.0)] * 6 + [(256, 256, 0.02)],
+            "many plain, one flat": big + [(2048, 4, 0.0)],
+            "many plain, one dense": [(4096, 4096, 0.0)] * 9 + [(512, 512, 0.02)],
+            "forced and dense": [(1024, 512, 1e-3)] * 8 + [(512, 512, 0.02)],
+            "one column": [(64, 65536, 1e-3)] * 10,
+            "two groups": [(64, 32, 1e-3)] * 300,
+            "forced, many": [(128, 64, 1e-3)] * 150}[kind]
+
+
+@pytest.mark.parametrize("kind,marches", [("all", {2: 1, 3: 1, 5: 1, 66: 1}), ("one dense", {2: 0, 3: 0, 5: 0, 66: 0}),
+                                          ("many plain, one flat", {2: 1, 3: 1, 5: 1, 66: 1}),
+                                          ("many plain, one dense", {2: 0, 3: 0, 5: 1, 66: 1}),
+                                          ("forced and dense", {2: 0, 3: 0, 5: 0, 66: 0}),
+                                          ("one column", {2: 0, 3: 0, 5: 0, 66: 0}),
+                                          ("two groups", {4: 1, 3: 0, 5: 0, 66: 0}),
+                                          ("forced, many", {2: 1, 3: 0, 5: 0, 66: 1})])
+def test_untuned_batches_march_where_it_pays(pkg, kind, marches):
+    """The route of every length of call (by its launches: single steps take one
+    a step) and the members' states against a batch of single steps."""
+    members = _mixed(kind)
+    arena = sum(pkg.Batch.lattice_bytes(w, h) for w, h, _ in members) + (32 << 20)
+    with pkg.Batch(arena) as a, pkg.Batch(arena) as b:
+        b.set_step_kernel(1)
+        b.set_temporal_block(1)
+        for x in (a, b):
+            for i, (w, h, p) in enumerate(members):
+                assert x.add(w, h, 50 + i, p) == i
+                x.init_random(i, 0.3)
+        for n, want in marches.items():
+            before = a.kernel_launches, b.kernel_launches
+            a.step(n)
+            b.step(n)
+            single = b.kernel_launches - before[1]
+            assert single == n
+            rest = any(h < 6 or p >= 0.01 for _, h, p in members)      # (steps of their own)
+            got = a.kernel_launches - before[0]
+            assert (got != n) == bool(want) if not rest or not want else got > n, (n, got)
+        a.synchronize()
+        b.synchronize()
+        for i in sorted({0, 1, len(members) // 2, len(members) - 2, len(members) - 1}):
+            assert a.time(i) == b.time(i) == sum(marches)
+            assert np.array_equal(a.get_state(i), b.get_state(i)), members[i]
