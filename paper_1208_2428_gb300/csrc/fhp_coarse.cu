@@ -223,7 +223,8 @@ cudaError_t launch_coarse_grain(const Geometry& g, const uint32_t* state, const 
         // for 32 and 64 nodes, whose few rows gain less than a cluster costs (4096 x
         // 4096: 8.2 us with, 6.3 without).
         int ctas = 1;
-        while (per == 1 && ctas < 8 && grid * ctas * 2 <= 304u && B % (64 * ctas) == 0) ctas *= 2;
+        const unsigned most = 2u * (unsigned)sm_count();
+        while (per == 1 && ctas < 8 && grid * ctas * 2 <= most && B % (64 * ctas) == 0) ctas *= 2;
         if (ctas > 1) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(grid * ctas);

@@ -55,6 +55,9 @@ inline uint32_t rest_rules_mask(const Geometry& g) { return g.rules == 1 ? 0u : 
 
 Geometry make_geometry(int W, int H);
 
+// SMs of the current device (0: unknown).
+int sm_count();
+
 // Arguments of one k = 1 step kernel launch.
 struct StepArgs {
     const uint32_t* __restrict__ src;    // 7 planes of S_t

@@ -7,9 +7,8 @@
 #include "fhp_march.cuh"
 
 namespace fhp {
-namespace {
 
-int march_sms() {
+int sm_count() {
     static std::mutex m;
     static int sms[64] = {};
     int dev = 0;
@@ -18,6 +17,8 @@ int march_sms() {
     if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     return sms[dev];
 }
+
+namespace {
 
 cudaError_t march_any(int k, const StepArgs& a, const MarchArgs& b, const MarchVariant& v, bool launch, int* n,
                       cudaStream_t s) {
@@ -33,7 +34,7 @@ cudaError_t march_resident(int k, const MarchVariant& v, int* warps) {
     int per_sm = 0;
     const cudaError_t e = march_any(k, StepArgs{}, MarchArgs{}, v, false, &per_sm, nullptr);
     if (e != cudaSuccess) return e;
-    *warps = march_sms() * per_sm * kMarchWarps;
+    *warps = sm_count() * per_sm * kMarchWarps;
     return *warps > 0 ? cudaSuccess : cudaErrorInvalidDevice;
 }
 
