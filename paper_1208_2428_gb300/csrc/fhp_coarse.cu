@@ -17,7 +17,8 @@
 // The latency of the loads bounds it, so 16 warps take two rows at a time, and
 // clusters share the rows of large blocks.  16384 x 4096, B = 64, from HBM:
 // 15.3 us; 23.5 us with 8 warps and one row at a time (and with words); 49 us
-// when one warp gathered the words of one block.  Repeated, in L2: B = 32 12.5
+// when one warp gathered the words of one block (which is left to narrow
+// lattices).  Repeated, in L2: B = 32 12.5
 // us, 64 8.4, 128 and more 10.4 (256 14.4 and 512 20.6 without clusters); 4096 x
 // 4096, B = 128 and more: 8.3 (10.3, 14.2, 20.6).
 #include <cooperative_groups.h>
@@ -207,12 +208,72 @@ __global__ void __launch_bounds__(kQuadBlock, 2) coarse_quads_kernel(Geometry g,
     write_cell((long long)by * nbx + bx, sum, counts, rho, ux, uy);
 }
 
+// A warp per block: for narrow lattices, whose rows leave the lanes of a CTA's
+// warps empty.
+template <bool SOLID>
+__global__ void __launch_bounds__(kBlock) coarse_warp_kernel(Geometry g, const uint32_t* __restrict__ state,
+                                                             const uint32_t* __restrict__ solid, int B, int Bw,
+                                                             long long cells, int32_t* __restrict__ counts,
+                                                             float* __restrict__ rho, float* __restrict__ ux,
+                                                             float* __restrict__ uy) {
+    const int lane = threadIdx.x & 31;
+    const int nbx = g.W / B;
+    const long long cell = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    if (cell >= cells) return;   // (a whole warp)
+    const int by = (int)(cell / nbx), bx = (int)(cell - (long long)by * nbx);
+    const size_t base = (size_t)by * B * g.Pq + (size_t)bx * Bw;
+    unsigned n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int i = lane; i < B * Bw; i += 32) {
+        const size_t off = base + (size_t)(i / Bw) * g.Pq + i % Bw;
+        const uint32_t f = SOLID ? ~solid[off] : 0xFFFFFFFFu;
+        n[7] += __popc(f);
+#pragma unroll
+        for (int k = 0; k < 7; ++k) n[k] += __popc(state[(size_t)k * g.plane_words + off] & f);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) n[k] = __reduce_add_sync(0xFFFFFFFFu, n[k]);
+    if (lane == 0) write_cell(cell, n, counts, rho, ux, uy);
+}
+
+// Where a warp per block is the faster (us, a warp per block / the kernels
+// above).  These give every row of blocks a CTA, whatever the row's length, so
+// what counts is how many rows of blocks there are for the SMs, and how few words
+// a row has: 120 rows of blocks of 64 8.3 / 6.5 at every width; 240 rows 8.3 / 10.2
+// with 8 words, 10.5 / 10.3 with 16; 1920 rows 10.4 / 37.1 with 2 words, 30.6 / 37.1
+// with 12, 39.3 / 37.1 with 16.  B = 32: 3840 rows of 1 word 14.5 / 49.4, of 5 words
+// 43.4 / 49.6, of 6 52.7 / 50.3, 120 rows 6.5 / 6.5.  B = 128: 120 rows 12.4 / 10.8,
+// 180 rows of 24 words 12.4 / 14.5, of 28 words 14.6 / 14.5, 960 rows of 28 words
+// 35.0 / 43.2, of 32 words 51.5 / 45.2.  B = 256: 240 rows 26.9 / 22.7, 480 rows of 16 words 26.9 / 39.2, of 24
+// words 39.2 / 41.2.  B = 96: 640 rows of 3 words 9.4 / 10.6, of 6 words 12.0 / 10.5,
+// 1280 rows of 6 words 14.6 / 16.5.  Not for larger blocks, whose words one warp
+// would take too long to walk (B = 512: 88 / 23).
+bool warp_per_block(const Geometry& g, int Bw) {
+    const int rows = g.H / (32 * Bw), sms = sm_count();
+    switch (Bw) {
+        case 1: return rows > sms && g.Wq <= 5;
+        case 2: return rows > sms && g.Wq <= 12;
+        case 3: return rows > sms && rows > 200 * g.Wq;
+        case 4: return rows > sms && g.Wq <= 28;
+        case 8: return 2 * rows > 5 * sms && g.Wq <= 24;
+        default: return false;
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_coarse_grain(const Geometry& g, const uint32_t* state, const uint32_t* solid,
                                 bool has_solid, int B, int32_t* counts, float* rho, float* ux,
                                 float* uy, cudaStream_t stream) {
     const int Bw = B / 32, nbx = g.W / B;
+    if (warp_per_block(g, Bw)) {
+        const long long cells = (long long)nbx * (g.H / B);
+        const unsigned grid = (unsigned)((cells + kWarps - 1) / kWarps);
+        auto launch = [&](auto kernel) {
+            kernel<<<grid, kBlock, 0, stream>>>(g, state, solid, B, Bw, cells, counts, rho, ux, uy);
+        };
+        has_solid ? launch(coarse_warp_kernel<true>) : launch(coarse_warp_kernel<false>);
+        return cudaGetLastError();
+    }
     if (Bw <= 2 || Bw % 4 == 0) {
         const int per = Bw <= 2 ? 4 / Bw : 1, lanes = Bw <= 2 ? 1 : Bw / 4;   // blocks per quad, quads per block
         const int width = per > 1 ? 32 : lanes * (lanes >= 32 ? 1 : 32 / lanes);

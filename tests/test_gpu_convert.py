@@ -62,6 +62,27 @@ def test_coarse_grain_blocks(pkg, oracle_mod, W, H, B, solid):
         np.testing.assert_allclose(g, r.astype(np.float32), rtol=1e-6, atol=1e-30)
 
 
+@pytest.mark.parametrize("W,H,B", [(32, 5120, 32), (160, 9600, 32), (192, 9600, 32), (384, 12800, 64), (96, 61440, 96),
+                                   (192, 122880, 96), (768, 23040, 128), (128, 19200, 128), (256, 98560, 256),
+                                   (512, 97024, 256), (1024, 23040, 128)])
+@pytest.mark.parametrize("solid", [False, True])
+def test_coarse_grain_narrow(pkg, oracle_mod, W, H, B, solid):
+    """Lattices of many short rows of blocks, on either side of the line from
+    which a warp takes a block."""
+    rng = np.random.Generator(np.random.PCG64(W + H + B))
+    s = rng.integers(0, 128, size=(H, W), dtype=np.uint8)
+    if solid:
+        s[rng.random((H, W)) < 0.3] |= 0x80
+        s[-B:, -B:] |= 0x80                    # a block without fluid nodes
+    with pkg.Lattice(W, H, seed=1) as lat:
+        lat.set_state(s)
+        got = lat.coarse_grain(B)
+    want = oracle_mod.coarse_grain(s, B)
+    assert np.array_equal(got[0], want[0])
+    for g, r in zip(got[1:], want[1:]):
+        np.testing.assert_allclose(g, r.astype(np.float32), rtol=1e-6, atol=1e-30)
+
+
 def test_coarse_grain_sparse_large_block(pkg, oracle_mod):
     """One block with more fluid nodes than a float counts (2^25 + 2) and few
     particles: the density is the quotient in doubles, rounded once."""
