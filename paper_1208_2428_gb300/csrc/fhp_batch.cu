@@ -1470,6 +1470,7 @@ int march_block(const fhp_batch* b) {
 //     to 1.8 with forcing, without it 1.6 for 4 steps and, in passes of 3, 0.88 for
 //     32).
 bool march_pays(const fhp_batch* b, int n) {
+    if (n < 2) return false;
     long long plain = 0, forced = 0, padded = 0, narrow = 0;
     int count = 0;
     bool rest = false, dense = false;
@@ -1487,7 +1488,7 @@ bool march_pays(const fhp_batch* b, int n) {
         padded += p;
         if (m.g.nq == 1) narrow += p;
     }
-    if (count == 0 || n < 2) return false;
+    if (count == 0) return false;
     if (rest) {
         if (dense) return forced == 0 && plain >= 150000000 && n >= 5;
         return plain + forced >= (forced ? 100000000 : 40000000);
