@@ -560,3 +560,22 @@ def test_fhp3_row_strips(fhp_mod, oracle_mod):
             st.close()
     want, _ = oracle_mod.run(s0, seed, 0, steps, p, rules=3)
     assert_same(got, want, "FHP-III strips")
+
+
+def test_cylinder_full_size_multi_step_and_marching(fhp_mod):
+    """16384 x 4096 cylinder at full size: the automatic choice marches, and it
+    and the multi-step ring agree with the direct kernel (which
+    test_cylinder_full_size compares with the oracle)."""
+    import torch
+    job = workloads.cylinder_16384x4096()
+    got = []
+    for kernel in (1, 3, 0):
+        with fhp_mod.Lattice(job.W, job.H, seed=job.seed, forcing_p=job.p, step_kernel=kernel) as lat:
+            lat.load_obstacle_shapes(workloads.cylinder_shapes(job.W, job.H))
+            lat.init_random(0.25)
+            assert lat.temporal_block_kernel == (3 if kernel == 0 else 0)
+            assert kernel == 0 or lat.step_kernel == kernel
+            lat.step(12)
+            got.append(lat.get_state_tensor())
+            lat.synchronize()
+    assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
