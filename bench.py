@@ -610,6 +610,10 @@ def run_gpu(args):
     # For the resident kernel the temporal block is the exchange interval
     # (steps between hand-offs of strip edge rows), not a blocked pass.
     resident = lat.step_kernel == 4
+    if args.rules == 3 and args.step_kernel in (0, 4) and lat.step_kernel == 3:
+        # FHP-III strips in shared memory are reported under the number of the
+        # multi-step kernel.
+        kernel_name = "fhp_resident_kernel if the strips fit shared memory, else fhp_run_kernel"
     if resident and k_block > 1:
         kernel_name = f"fhp_resident_kernel (exchange every {k_block} steps)"
     elif k_block > 1:

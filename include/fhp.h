@@ -202,10 +202,13 @@ FHP_API int fhp_load_obstacle_shapes(fhp_lattice* lattice, const fhp_shape* shap
  * states turn their movers by +-60 degrees (chirality), two-state classes
  * swap, and the three-state classes of momentum c_k cycle (chirality sets the
  * direction); it keeps every FHP-II collision.  FHP-III lattices step with
- * the direct, bulk-copy ring and multi-step ring kernels (step kernels 1-3;
- * kernel 4 and temporal blocks k > 1 fall back to those; the automatic choice
- * and kernel 4 keep a lattice that fits in shared memory for the steps of a
- * call, reported as kernel 3) and cannot be batch members.  Takes effect from the next step.
+ * the direct, bulk-copy ring and multi-step ring kernels (step kernels 1-3), with
+ * register marching where that is the automatic choice, and, where the automatic
+ * choice or kernel 4 finds room for their strips in shared memory, with the
+ * resident kernel (an exchange every step), which fhp_get_step_kernel and
+ * fhp_autotune report as 3: all steps of a call in one launch.  Kernel 4 without
+ * room and temporal blocks k > 1 fall back to kernels 1-3.  FHP-III lattices
+ * cannot be batch members.  Takes effect from the next step.
  * FHP_EINVAL for other values. */
 #define FHP_RULES_FHP_I 1
 #define FHP_RULES_FHP_II 2
