@@ -115,7 +115,8 @@ cudaError_t launch_resident(const Geometry& g, uint32_t* buf0, uint32_t* buf1, c
     a.ft = ft;
     ResArgs ra;
     ra.buf0 = buf0;
-    ra.out = resident_flips(nsteps, gh) ? buf1 : buf0;
+    ra.buf1 = buf1;
+    ra.flip = resident_flips(nsteps, gh);
     ra.halo = halo;
     ra.nsteps = nsteps;
     ra.t0 = t0;

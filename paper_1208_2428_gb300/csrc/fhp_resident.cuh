@@ -49,10 +49,11 @@ constexpr int kResSmemLimit = 224 * 1024;
 constexpr int kLoneQuads = 160;
 
 struct ResArgs {
-    const uint32_t* buf0;  // state at t0
-    uint32_t* out;         // the result: buf0 only if strips exchange rows before they store (resident_flips)
+    uint32_t* buf0;        // state at t0
+    uint32_t* buf1;
     uint32_t* halo;        // exchanged units of 32 bytes: [2 slots][G][2 sides][units][nq], zero at launch
     int nsteps;
+    int flip;              // the result goes to buf1 (resident_flips), else to buf0
     unsigned long long t0;
     int nmax;              // most rows any CTA owns
     unsigned long long nq_magic;   // ceil(2^32 / nq): j / nq == (j * nq_magic) >> 32 for small j
@@ -339,9 +340,10 @@ __global__ void __launch_bounds__(kRes1Threads, 1) fhp_resident_kernel(const Ste
     }
     // The owned rows of the final state.
     const uint32_t* fin = X + (ra.nsteps & 1 ? half : 0);
+    uint32_t* out = ra.flip ? ra.buf1 : ra.buf0;
     for (int i = tid; i < 7 * n * q4; i += T) {
         const int p = i / (n * q4), rem = i - p * n * q4, rr = rem / q4, w = 4 * (rem % q4);
-        st4(ra.out + (size_t)p * a.plane_words + (size_t)(y0 + rr) * Pq + w,
+        st4(out + (size_t)p * a.plane_words + (size_t)(y0 + rr) * Pq + w,
             ld4(fin + p * pstride + (rr + GH) * Pq + w));
     }
 }
