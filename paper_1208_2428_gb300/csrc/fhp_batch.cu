@@ -1557,16 +1557,22 @@ int launch_march_passes(fhp_batch* b, int k, const std::vector<int>& passes) {
         t.err = b->d_err;
         // The counters are not cleared between launches: a launch's passes
         // count on from where the counters can be (and once in 2^31 passes
-        // they start again).
+        // they start again).  A captured launch runs whenever its graph does,
+        // with the epoch it was captured with: it clears them itself.
         int longest = 0;
         for (size_t i : group) longest = std::max(longest, passes[i]);
-        if (b->march_epoch > 0x7FFFFFFFu - (unsigned int)longest) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(b->stream, &capture);
+        if (e != cudaSuccess) return bcuda(b, e, "asking whether the stream is captured");
+        const bool captured = capture != cudaStreamCaptureStatusNone;
+        if (captured || b->march_epoch > 0x7FFFFFFFu - (unsigned int)longest) {
             e = cudaMemsetAsync(b->d_march_flags, 0, kMarchFlagBytes, b->stream);
             if (e != cudaSuccess) return bcuda(b, e, "clearing the pass counters");
-            b->march_epoch = 0;
+            if (!captured) b->march_epoch = 0;
         }
-        t.epoch = b->march_epoch;
-        b->march_epoch += (unsigned int)longest;
+        t.epoch = captured ? 0u : b->march_epoch;
+        b->march_epoch = captured ? std::max(b->march_epoch, (unsigned int)longest)
+                                  : b->march_epoch + (unsigned int)longest;
         int cta = 0;
         for (size_t j = 0; j < group.size(); ++j) {
             const Member& m = b->members[group[j]];

@@ -243,3 +243,44 @@ def test_untuned_batches_march_where_it_pays(pkg, kind, marches):
         for i in sorted({0, 1, len(members) // 2, len(members) - 2, len(members) - 1}):
             assert a.time(i) == b.time(i) == sum(marches)
             assert np.array_equal(a.get_state(i), b.get_state(i)), members[i]
+
+
+def test_captured_batch_step_replays(pkg):
+    """A captured call of a batch that has marched before, replayed: its passes
+    wait for one another at every replay, and calls between and after the replays
+    are not disturbed."""
+    import torch
+    stream = torch.cuda.Stream()
+    members = [(2048, 1536), (512, 300), (4160, 512), (96, 2000)]
+    arena = sum(pkg.Batch.lattice_bytes(w, h) for w, h in members) + (32 << 20)
+    with pkg.Batch(arena, stream=stream) as a, pkg.Batch(arena, stream=stream) as b:
+        b.set_step_kernel(1)
+        b.set_temporal_block(1)
+        for x in (a, b):
+            for i, (w, h) in enumerate(members):
+                x.add(w, h, 70 + i, 0.0)
+                x.init_random(i, 0.3)
+            x.step(18)                     # (an even number of passes, as below)
+            x.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        launches = a.kernel_launches
+        with torch.cuda.graph(graph, stream=stream):
+            a.step(12)                     # the graph: steps 18 .. 29, from and to the same buffers
+        assert a.kernel_launches - launches == 1
+        with torch.cuda.stream(stream):
+            for _ in range(3):
+                graph.replay()
+                a.step(6)                  # steps 30 .. 35, 36 .. 41, 42 .. 47
+            graph.replay()
+        for start in (30, 36, 42, None):
+            for i in range(len(members)):
+                b.set_time(i, 18)
+            b.step(12)
+            if start is not None:
+                for i in range(len(members)):
+                    b.set_time(i, start)
+                b.step(6)
+        a.synchronize()
+        b.synchronize()
+        for i in range(len(members)):
+            assert np.array_equal(a.get_state(i), b.get_state(i)), members[i]
