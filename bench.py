@@ -112,11 +112,13 @@ def source_hash(files=("fhp_step.cu", "fhp_device.cuh", "fhp_quad.cuh")) -> str:
     return h.hexdigest()[:16]
 
 
-def recorded_traffic(workload_name: str, steps_per_launch: float):
-    """DRAM bytes per launch of the step kernel from the committed ncu summary
-    (recorded per lattice step of the workload), if it was taken on the
-    current kernel source."""
-    path = os.path.join(ROOT, "profiles", f"fhp_step_{workload_name}.txt")
+def recorded_traffic(workload_name: str, steps_per_launch: float, march: bool = False):
+    """DRAM bytes per launch of the step kernel (the multi-step ring, or with
+    ``march`` register marching) from the committed ncu summary (recorded per
+    lattice step of the workload), if it was taken on the current kernel
+    source."""
+    path = os.path.join(ROOT, "profiles", f"fhp_{'march' if march else 'step'}_{workload_name}.txt")
+    sources = ("fhp_march.cuh", "fhp_device.cuh", "fhp_quad.cuh", "fhp_rules.cuh")
     try:
         fields = {}
         with open(path) as f:
@@ -124,7 +126,7 @@ def recorded_traffic(workload_name: str, steps_per_launch: float):
                 if ":" in line:
                     k, v = line.split(":", 1)
                     fields[k.strip()] = v.strip()
-        if fields.get("source_hash") != source_hash():
+        if fields.get("source_hash") != (source_hash(sources) if march else source_hash()):
             return None
         return float(fields["dram_bytes_per_lattice_step_full_size"]) * steps_per_launch
     except Exception:
@@ -641,8 +643,10 @@ def run_gpu(args):
     bytes_per_launch = bytes_per_node * nodes * steps_per_launch / k_pass
     achieved = bytes_per_launch / launch_s / 1e9
     peak, peak_src = measured_hbm_peak()
-    # The committed capture is of the multi-step kernel.
-    traffic = recorded_traffic(job.name, steps_per_launch) if (lat.step_kernel == 3 and k_block == 1) else None
+    # The committed captures are of register marching (k = 2) and of the multi-step kernel.
+    march = lat.temporal_block_kernel == 3 and k_block == 2
+    traffic = (recorded_traffic(job.name, steps_per_launch, march)
+               if march or (lat.step_kernel == 3 and k_block == 1) else None)
 
     # End to end through the C ABI with host buffers: pinned initial state in,
     # coarse-grained fields out, host<->device copies inside the timed region.

@@ -143,10 +143,10 @@ class Server:
         self.batch.set_graph_steps(graph_steps)
         # Temporal block of the batch: quanta (8..64 steps) are too short for a
         # tuning trial that includes blocked passes (six parts of at least 16
-        # steps), so it is set here -- 1 (no blocking, the default) or 2 / 4
-        # (blocked passes for the lattices narrow enough, the rest of each
-        # quantum on the step kernel); the kernel and tile size are still tuned
-        # online within a quantum.
+        # steps), so it is set here -- 1 (single steps, the default; a batch whose
+        # block is automatic would march instead) or 2 / 4 (blocked passes for the
+        # lattices narrow enough, the rest of each quantum on the step kernel); the
+        # kernel and tile size are still tuned online within a quantum.
         if hasattr(self.batch, "set_temporal_block"):
             self.batch.set_temporal_block(int(temporal_block))
         self.hbm_budget = int(hbm_budget)
